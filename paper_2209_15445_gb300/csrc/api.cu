@@ -115,6 +115,7 @@ struct adept_ctx {
   float2 *g32 = nullptr, *e32 = nullptr, *p32 = nullptr;
   double *re64 = nullptr, *rp64 = nullptr, *Tc = nullptr, *kc = nullptr;
   float *re32 = nullptr, *rp32 = nullptr;
+  uint16_t* xr[4] = {nullptr, nullptr, nullptr, nullptr};  // range indexes: e-, e+ FP64, e-, e+ FP32
   TrackIn* stage = nullptr;
   uint32_t* stage_meta = nullptr;
   uint32_t* stage_keys = nullptr;
@@ -371,6 +372,7 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   ok = ok && carve_n(cp, &c->g64, nn * kNTabG) && carve_n(cp, &c->e64, nn * kNTabE) && carve_n(cp, &c->p64, nn * kNTabP);
   ok = ok && carve_n(cp, &c->g32, nn * kNTabG) && carve_n(cp, &c->e32, nn * kNTabE) && carve_n(cp, &c->p32, nn * kNTabP);
   ok = ok && carve_n(cp, &c->re64, nn) && carve_n(cp, &c->rp64, nn) && carve_n(cp, &c->re32, nn) && carve_n(cp, &c->rp32, nn);
+  for (int k = 0; k < 4; ++k) ok = ok && carve_n(cp, &c->xr[k], (size_t)kRangeKeys * n_materials);
   ok = ok && carve_n(cp, &c->Tc, kMaxMat) && carve_n(cp, &c->kc, kMaxMat);
   EventView& E = P.evt;
   const uint32_t ms = o.max_events;
@@ -416,7 +418,8 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   P.geo.half_xy = geometry->transverse_half_mm; P.geo.half_z = geometry->half_length_mm;
   P.geo.bnd = bnd; P.geo.vol_mat = vm; P.geo.vol_bin = vb;
   P.mat = c->mat_dev;
-  P.tab = TableView{c->g64, c->e64, c->p64, c->g32, c->e32, c->p32, c->re64, c->rp64, c->re32, c->rp32, c->Tc, c->kc};
+  P.tab = TableView{c->g64, c->e64, c->p64, c->g32, c->e32, c->p32, c->re64, c->rp64, c->re32, c->rp32,
+                    c->xr[0], c->xr[1], c->xr[2], c->xr[3], c->Tc, c->kc};
   E.max_slots = ms;
   P.max_log = o.max_generation_log;
   P.field_T = cuts->field_T;
@@ -502,9 +505,9 @@ extern "C" int adept_build_tables(adept_ctx* c) {
   const std::vector<double>& in = c->mat_rec;
   CK(cudaMemcpyAsync(c->mat_in, in.data(), sizeof(double) * in.size(), cudaMemcpyHostToDevice, c->stream));
   CK(launch_build_tables(c->P, c->mat_in, c->n_mat, c->range_cut, c->mat_dev, c->scratch, c->g64, c->e64, c->p64,
-                         c->g32, c->e32, c->p32, c->re64, c->rp64, c->re32, c->rp32, c->Tc, c->kc, c->stream));
+                         c->g32, c->e32, c->p32, c->re64, c->rp64, c->re32, c->rp32, c->xr, c->Tc, c->kc, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  c->stats.launches += 6;
+  c->stats.launches += 7;
   c->built = true;
   return ADEPT_OK;
 }

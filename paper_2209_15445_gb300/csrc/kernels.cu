@@ -144,10 +144,35 @@ __global__ void k_pack(const MatDev* mats, int n_mat, BuildScratch s, PackOut o,
   o.rp32[r] = (float)v[V_RP * kNNode + i];
 }
 
+// The range index of inverse_range: one thread per key of one material's node row, blockIdx.y
+// the row (e- FP64, e+ FP64, e- FP32, e+ FP32).
+__device__ __forceinline__ float key_edge(float n0, int k) { return __uint_as_float((uint32_t)(range_key(n0) + k) << 19); }
+__device__ __forceinline__ double key_edge(double n0, int k) { return __hiloint2double((range_key(n0) + k) << 16, 0); }
+template <class R>
+__device__ __forceinline__ uint16_t index_entry(const R* nodes, int k) {
+  const R edge = key_edge(nodes[0], k);
+  int lo = 0, hi = kNNode - 1;  // the last node at or below the edge, at most the last interval's
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (nodes[mid] <= edge) lo = mid; else hi = mid;
+  }
+  return (uint16_t)lo;
+}
+struct IndexOut {
+  uint16_t* x[4];
+};
+__global__ void k_range_index(int n_mat, PackOut o, IndexOut x) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n_mat * kRangeKeys) return;
+  const int m = idx / kRangeKeys, k = idx % kRangeKeys, row = blockIdx.y;
+  if (row < 2) x.x[row][idx] = index_entry((row ? o.rp64 : o.re64) + m * kNNode, k);
+  else x.x[row][idx] = index_entry((row == 3 ? o.rp32 : o.re32) + m * kNNode, k);
+}
+
 cudaError_t launch_build_tables(const Params& P, const double* mat_in, int n_mat, double range_cut, MatDev* mat,
                                 BuildScratch s, double2* g64, double2* e64, double2* p64, float2* g32,
                                 float2* e32, float2* p32, double* re64, double* rp64, float* re32, float* rp32,
-                                double* Tc, double* kc, cudaStream_t st) {
+                                uint16_t* const range_index[4], double* Tc, double* kc, cudaStream_t st) {
   const int nn = n_mat * kNNode;
   const int B = 128;
   k_materials<<<1, 32, 0, st>>>(mat_in, n_mat, mat);
@@ -157,6 +182,8 @@ cudaError_t launch_build_tables(const Params& P, const double* mat_in, int n_mat
   k_ranges<<<1, 32, 0, st>>>(mat, n_mat, s);
   PackOut o{g64, e64, p64, g32, e32, p32, re64, rp64, re32, rp32};
   k_pack<<<(nn + B - 1) / B, B, 0, st>>>(mat, n_mat, s, o, P.process_mask);
+  const IndexOut x{{range_index[0], range_index[1], range_index[2], range_index[3]}};
+  k_range_index<<<dim3((n_mat * kRangeKeys + B - 1) / B, 4), B, 0, st>>>(n_mat, o, x);
   return cudaGetLastError();
 }
 
@@ -483,7 +510,8 @@ template <class R>
 __global__ void k_probe_inverse_range(Params P, int s, int m, const double* Rv, int n, double* out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  out[i] = inverse_range<R>(range_nodes<R>(P.tab, s == 2) + (size_t)m * kNNode, (R)Rv[i], kNNode - 2);
+  out[i] = inverse_range<R>(range_nodes<R>(P.tab, s == 2) + m * kNNode, range_index<R>(P.tab, s == 2) + m * kRangeKeys,
+                            (R)Rv[i]);
 }
 
 cudaError_t launch_probe_inverse_range(const Params& P, int s, int m, int prec, const double* R, int n, double* out,
@@ -604,7 +632,9 @@ __global__ void k_probe_continuous(Params P, int which, int species, int m, doub
                                   : tab_e<R>(P.tab) + ((size_t)m * kNNode + bin) * kNTabE);
   const R Rr = lerp_rec<R>(rec, 1, tt);
   R Epr = 0;
-  if ((R)s < Rr) Epr = inverse_range<R>(range_nodes<R>(P.tab, species == 2) + (size_t)m * kNNode, Rr - (R)s, bin + 1);
+  if ((R)s < Rr)
+    Epr = inverse_range<R>(range_nodes<R>(P.tab, species == 2) + m * kNNode,
+                           range_index<R>(P.tab, species == 2) + m * kRangeKeys, Rr - (R)s);
   const double Ep = (Epr > (R)T) ? T : to_d<R>(Epr);
   const R xi = (R)(kTwoPiRe2Me * md.n_el);
   const R sig = M<R>::sqrt(fluct_sigma2<R>((R)T, xi, (R)P.tab.Tc[m], (R)s, species == 2));

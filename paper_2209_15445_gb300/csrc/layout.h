@@ -14,6 +14,7 @@ constexpr int kNTabG = 3;     // gamma: compton, pair, photo
 constexpr int kNTabE = 4;     // e-: dedx, range, ioni, brem
 constexpr int kNTabP = 5;     // e+: dedx, range, ioni, brem, annihilation
 constexpr int kMaxLogGen = 1 << 16;
+constexpr int kRangeKeys = 768;  // keys of the range index: 16 an octave over 48 octaves
 
 struct GeoView {
   int kind;          // 0 slab, 1 tubes
@@ -48,6 +49,9 @@ struct TableView {
   // range nodes for the inversion: [mat][node]
   const double* re64; const double* rp64;
   const float* re32; const float* rp32;
+  // for each key of a range, the node interval it falls in: [mat][kRangeKeys] (inverse_range)
+  const uint16_t* xe64; const uint16_t* xp64;
+  const uint16_t* xe32; const uint16_t* xp32;
   // production thresholds per material
   const double* Tc; const double* kc;
 };
@@ -171,7 +175,8 @@ struct BuildScratch {
 cudaError_t launch_build_tables(const Params& P, const double* mat_in, int n_mat, double range_cut,
                                 MatDev* mat, BuildScratch s, double2* g64, double2* e64, double2* p64,
                                 float2* g32, float2* e32, float2* p32, double* re64, double* rp64,
-                                float* re32, float* rp32, double* Tc, double* kc, cudaStream_t st);
+                                float* re32, float* rp32, uint16_t* const range_index[4], double* Tc, double* kc,
+                                cudaStream_t st);
 // A tail chunk runs its generations as the body of a conditional (while) graph node, one
 // generation per iteration, until the queues are empty or a cap is reached; its kernels are
 // launched with gk = kGkDevice and read their place in the chunk from Ctrl::tail_k.

@@ -101,6 +101,10 @@ template <class R> __device__ __forceinline__ const R* range_nodes(const TableVi
 template <> __device__ __forceinline__ const double* range_nodes<double>(const TableView& T, bool pos) { return pos ? T.rp64 : T.re64; }
 template <> __device__ __forceinline__ const float* range_nodes<float>(const TableView& T, bool pos) { return pos ? T.rp32 : T.re32; }
 
+template <class R> __device__ __forceinline__ const uint16_t* range_index(const TableView& T, bool pos);
+template <> __device__ __forceinline__ const uint16_t* range_index<double>(const TableView& T, bool pos) { return pos ? T.xp64 : T.xe64; }
+template <> __device__ __forceinline__ const uint16_t* range_index<float>(const TableView& T, bool pos) { return pos ? T.xp32 : T.xe32; }
+
 enum Outcome { kDead = 0, kAlive = 1, kInteract = 2 };
 
 // Phase A of one step of one track of species S (0 gamma, 1 e-, 2 e+) -- paper Sec. 3:
@@ -236,7 +240,9 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
   // that mean for a track that survives the mean loss
   if (q != 0 && m >= 0) {
     R Epr = 0;
-    if (s < Rr) Epr = inverse_range<R>(range_nodes<R>(P.tab, S == 2) + (size_t)m * kNNode, Rr - s, bin + 1);
+    if (s < Rr)
+      Epr = inverse_range<R>(range_nodes<R>(P.tab, S == 2) + m * kNNode, range_index<R>(P.tab, S == 2) + m * kRangeKeys,
+                             Rr - s);
     double Ep = (Epr > Er) ? t.E : to_d<R>(Epr);
     if constexpr (PH) {
       if (fluct && s < Rr && Ep >= P.tcut) {
