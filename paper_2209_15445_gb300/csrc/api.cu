@@ -275,18 +275,7 @@ static int build_geometry(adept_ctx* c, const adept_geometry* g) {
   return ADEPT_OK;
 }
 
-static size_t track_bytes(int precision) {
-  return 3 * 8 + 3 * (precision ? 4 : 8) + 8 + 8 + 3 * 4;
-}
-
-static bool carve_queue(adept_ctx* c, TrackSoA* q, uint32_t cap) {
-  *q = TrackSoA{};
-  if (c->opt.precision)  // split form: four arrays of 16-byte vectors
-    return carve_n(c, &q->xy, cap) && carve_n(c, &q->zE, cap) && carve_n(c, &q->un, cap) && carve_n(c, &q->meta, cap);
-  return carve_n(c, &q->x, cap) && carve_n(c, &q->y, cap) && carve_n(c, &q->z, cap) && carve_n(c, &q->ux, cap) &&
-         carve_n(c, &q->uy, cap) && carve_n(c, &q->uz, cap) && carve_n(c, &q->E, cap) && carve_n(c, &q->id, cap) &&
-         carve_n(c, &q->ev, cap) && carve_n(c, &q->step, cap) && carve_n(c, &q->nav, cap);
-}
+static size_t tile_bytes(int precision) { return precision ? Tile<float>::kBytes : Tile<double>::kBytes; }
 
 extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const adept_material* materials,
                           int32_t n_materials, const adept_cuts* cuts, const adept_options* options, void* dev_arena,
@@ -372,7 +361,10 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   ok = ok && carve_n(cp, &c->g64, nn * kNTabG) && carve_n(cp, &c->e64, nn * kNTabE) && carve_n(cp, &c->p64, nn * kNTabP);
   ok = ok && carve_n(cp, &c->g32, nn * kNTabG) && carve_n(cp, &c->e32, nn * kNTabE) && carve_n(cp, &c->p32, nn * kNTabP);
   ok = ok && carve_n(cp, &c->re64, nn) && carve_n(cp, &c->rp64, nn) && carve_n(cp, &c->re32, nn) && carve_n(cp, &c->rp32, nn);
-  for (int k = 0; k < 4; ++k) ok = ok && carve_n(cp, &c->xr[k], (size_t)kRangeKeys * n_materials);
+  // the range indexes take the place of the bin integrals, which only the build reads
+  static_assert(4 * kRangeKeys * sizeof(uint16_t) <= 3 * kNNode * sizeof(double), "range indexes");
+  for (int k = 0; k < 4; ++k)
+    c->xr[k] = reinterpret_cast<uint16_t*>(c->scratch.bins) + (size_t)k * kRangeKeys * n_materials;
   ok = ok && carve_n(cp, &c->Tc, kMaxMat) && carve_n(cp, &c->kc, kMaxMat);
   EventView& E = P.evt;
   const uint32_t ms = o.max_events;
@@ -381,8 +373,6 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   ok = ok && carve_n(cp, &P.gen_log, 3 * (size_t)o.max_generation_log);
   unsigned long long* steplen = nullptr;
   ok = ok && carve_n(cp, &steplen, 3 * 64);
-  TrackSoA* qdesc = nullptr;
-  ok = ok && carve_n(cp, &qdesc, 6);
   ok = ok && carve_n(cp, &P.leak, o.max_outgoing);
   P.leak_cap = o.max_outgoing;
   c->probe_bytes = (size_t)8 << 20;
@@ -390,7 +380,7 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   ok = ok && c->probe;
   if (!ok) return ADEPT_ENOMEM;
   // the remainder: primary staging (1/16, at least room for 4096 tracks) and the queues
-  const size_t per_track = track_bytes(o.precision);
+  const size_t per_track = tile_bytes(o.precision) / 32;
   size_t rest = c->arena_bytes - ((c->arena_used + 255) & ~(size_t)255);
   size_t stage_cap = std::max<size_t>(4096, rest / 16 / (sizeof(TrackIn) + 12));
   stage_cap = std::min<size_t>(stage_cap, (size_t)1 << 22);
@@ -399,8 +389,10 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   if (!ok) return ADEPT_ENOMEM;
   c->stage_cap = stage_cap;
   rest = c->arena_bytes - ((c->arena_used + 255) & ~(size_t)255);
-  // 6 queues x 11 arrays, each padded to 256 bytes
-  uint64_t cap = rest > 6 * 11 * 256 ? (rest - 6 * 11 * 256) / (6 * per_track) : 0;
+  // six queues of whole tiles, each padded to 256 bytes
+  constexpr size_t kPad = 11 * 256;
+  static_assert(31 * (Tile<double>::kBytes / 32) + 255 <= kPad, "a queue's padding");
+  uint64_t cap = rest > 6 * kPad ? (rest - 6 * kPad) / (6 * per_track) : 0;
   if (o.track_capacity) {
     if (o.track_capacity > cap) return ADEPT_ENOMEM;
     cap = o.track_capacity;
@@ -408,11 +400,11 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   cap = std::min<uint64_t>(cap, 0xFFFFFFF0ull);
   if (cap < 1024) return ADEPT_ENOMEM;
   o.track_capacity = cap;
-  for (int par = 0; par < 2; ++par)
-    for (int s = 0; s < 3; ++s)
-      if (!carve_queue(cp, &P.q[par][s], (uint32_t)cap)) return ADEPT_ENOMEM;
+  P.queue_bytes = ((cap + 31) / 32 * tile_bytes(o.precision) + 255) & ~(size_t)255;
+  P.queues = static_cast<char*>(carve(cp, 6 * P.queue_bytes));
+  if (!P.queues) return ADEPT_ENOMEM;
+  P.split = o.precision;
   P.cap = (uint32_t)cap;
-  P.qd = qdesc;
   // views
   P.geo.kind = c->kind; P.geo.n_vol = c->n_vol; P.geo.n_bins = c->n_bins;
   P.geo.half_xy = geometry->transverse_half_mm; P.geo.half_z = geometry->half_length_mm;
@@ -441,7 +433,6 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
     CK(cudaMemcpyAsync(vm, c->vol_mat.data(), sizeof(int) * c->n_vol, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(vb, c->vol_bin.data(), sizeof(int) * c->n_vol, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemsetAsync(P.ctrl, 0, sizeof(Ctrl), c->stream));
-    CK(cudaMemcpyAsync(qdesc, &P.q[0][0], sizeof(TrackSoA) * 6, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemsetAsync(steplen, 0, sizeof(unsigned long long) * 3 * 64, c->stream));
     CK(cudaMemsetAsync(E.state, 0, sizeof(uint32_t) * ms, c->stream));
     // the chunk status buffers are mapped: the finish pass writes them and the chunk's first

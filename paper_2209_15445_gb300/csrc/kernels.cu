@@ -182,6 +182,7 @@ cudaError_t launch_build_tables(const Params& P, const double* mat_in, int n_mat
   k_ranges<<<1, 32, 0, st>>>(mat, n_mat, s);
   PackOut o{g64, e64, p64, g32, e32, p32, re64, rp64, re32, rp32};
   k_pack<<<(nn + B - 1) / B, B, 0, st>>>(mat, n_mat, s, o, P.process_mask);
+  // (last: the index takes the place of the bin integrals)
   const IndexOut x{{range_index[0], range_index[1], range_index[2], range_index[3]}};
   k_range_index<<<dim3((n_mat * kRangeKeys + B - 1) / B, 4), B, 0, st>>>(n_mat, o, x);
   return cudaGetLastError();
@@ -303,7 +304,7 @@ __global__ void k_init_primaries(Params P, const TrackIn* recs, const uint32_t* 
     atomicAdd(P.evt.killed + slot, r.E + rest);
     return;
   }
-  store_track<R>(P.q[p][sp], d, r.pos[0], r.pos[1], r.pos[2], (R)r.dir[0], (R)r.dir[1], (R)r.dir[2], r.E,
+  store_track<R>(track_queue(P, p, sp), d, r.pos[0], r.pos[1], r.pos[2], (R)r.dir[0], (R)r.dir[1], (R)r.dir[2], r.E,
                  (unsigned long long)id, slot, 0u, (uint32_t)vol);
 }
 
@@ -345,8 +346,7 @@ __global__ void k_mark(Params P) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     const int sp = i < n0 ? 0 : (i < n0 + n1 ? 1 : 2);
     const uint32_t j = sp == 0 ? i : (sp == 1 ? i - n0 : i - n0 - n1);
-    const TrackSoA& q = P.q[p][sp];
-    const uint32_t ev = q.meta ? q.meta[j].z : q.ev[j];
+    const uint32_t ev = track_event(P, track_queue(P, p, sp), j);
     if (P.evt.alive[ev] != gen) P.evt.alive[ev] = gen;
   }
 }
@@ -372,8 +372,7 @@ __global__ void k_mark_bits(Params P) {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
       const int sp = i < n0 ? 0 : (i < n0 + n1 ? 1 : 2);
       const uint32_t j = sp == 0 ? i : (sp == 1 ? i - n0 : i - n0 - n1);
-      const TrackSoA& q = P.q[p][sp];
-      const uint32_t ev = q.meta ? q.meta[j].z : q.ev[j];
+      const uint32_t ev = track_event(P, track_queue(P, p, sp), j);
       if (P.evt.alive[ev] != gen) P.evt.alive[ev] = gen;
     }
     return;
@@ -384,8 +383,7 @@ __global__ void k_mark_bits(Params P) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     const int sp = i < n0 ? 0 : (i < n0 + n1 ? 1 : 2);
     const uint32_t j = sp == 0 ? i : (sp == 1 ? i - n0 : i - n0 - n1);
-    const TrackSoA& q = P.q[p][sp];
-    const uint32_t ev = q.meta ? q.meta[j].z : q.ev[j];
+    const uint32_t ev = track_event(P, track_queue(P, p, sp), j);
     if (ev < P.evt.max_slots) atomicOr(&seen[ev >> 5], 1u << (ev & 31u));
   }
   __syncthreads();

@@ -2,10 +2,6 @@
 // (kernels.cu, variants.cu) and the one-kernel-per-generation form (fused.cu): track load
 // and store, phase A (S1-S8), phase B (S9), scoring (S10), warp-aggregated appends and
 // the per-warp ring of deferred interactions.
-//
-// Queue descriptors are read from P.qd (device memory) with a runtime parity index:
-// indexing the kernel-parameter copy P.q that way makes the compiler copy the parameter
-// block to local memory once several species paths share a kernel.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -22,24 +18,40 @@ template <class R> struct Trk {
   uint32_t ev, step, nav;
 };
 
+// the queue of species s in the buffers of parity p
+__device__ __forceinline__ char* track_queue(const Params& P, int p, int s) {
+  return P.queues + (size_t)(3 * p + s) * P.queue_bytes;
+}
+// event slot of track i of a queue
+__device__ __forceinline__ uint32_t track_event(const Params& P, const char* q, uint32_t i) {
+  return P.split ? *(const uint32_t*)(q + (size_t)(i >> 5) * Tile<float>::kBytes + Tile<float>::kMeta + (i & 31u) * 16u + 8u)
+                 : *(const uint32_t*)(q + (size_t)(i >> 5) * Tile<double>::kBytes + Tile<double>::kEv + (i & 31u) * 4u);
+}
+
 // Queue loads are streaming (ld.global.cs): each slot is read once per generation.
 template <class R>
-__device__ __forceinline__ void load_track(const TrackSoA& q, uint32_t i, Trk<R>& t);
+__device__ __forceinline__ void load_track(const char* q, uint32_t tile, uint32_t lane, Trk<R>& t);
 template <>
-__device__ __forceinline__ void load_track<double>(const TrackSoA& q, uint32_t i, Trk<double>& t) {
-  t.x = __ldcs(q.x + i); t.y = __ldcs(q.y + i); t.z = __ldcs(q.z + i);
-  t.u[0] = __ldcs(q.ux + i); t.u[1] = __ldcs(q.uy + i); t.u[2] = __ldcs(q.uz + i);
-  t.E = __ldcs(q.E + i);
-  t.id = __ldcs(q.id + i);
-  t.ev = __ldcs(q.ev + i);
-  t.step = __ldcs(q.step + i);
-  t.nav = __ldcs(q.nav + i);
+__device__ __forceinline__ void load_track<double>(const char* q, uint32_t tile, uint32_t lane, Trk<double>& t) {
+  using L = Tile<double>;
+  const char* a = q + (size_t)tile * L::kBytes;
+  const double* d = (const double*)a + lane;
+  const uint32_t* w = (const uint32_t*)(a + L::kEv) + lane;
+  t.x = __ldcs(d + L::kX / 8); t.y = __ldcs(d + L::kY / 8); t.z = __ldcs(d + L::kZ / 8);
+  t.u[0] = __ldcs(d + L::kUX / 8); t.u[1] = __ldcs(d + L::kUY / 8); t.u[2] = __ldcs(d + L::kUZ / 8);
+  t.E = __ldcs(d + L::kE / 8);
+  t.id = __ldcs((const unsigned long long*)d + L::kId / 8);
+  t.ev = __ldcs(w);
+  t.step = __ldcs(w + (L::kStep - L::kEv) / 4);
+  t.nav = __ldcs(w + (L::kNav - L::kEv) / 4);
 }
 template <>
-__device__ __forceinline__ void load_track<float>(const TrackSoA& q, uint32_t i, Trk<float>& t) {
-  const double2 a = __ldcs(q.xy + i), b = __ldcs(q.zE + i);
-  const float4 c = __ldcs(q.un + i);
-  const uint4 d = __ldcs(q.meta + i);
+__device__ __forceinline__ void load_track<float>(const char* q, uint32_t tile, uint32_t lane, Trk<float>& t) {
+  using L = Tile<float>;
+  const char* r = q + (size_t)tile * L::kBytes + lane * 16u;
+  const double2 a = __ldcs((const double2*)(r + L::kXY)), b = __ldcs((const double2*)(r + L::kZE));
+  const float4 c = __ldcs((const float4*)(r + L::kUN));
+  const uint4 d = __ldcs((const uint4*)(r + L::kMeta));
   t.x = a.x; t.y = a.y; t.z = b.x; t.E = b.y;
   t.u[0] = c.x; t.u[1] = c.y; t.u[2] = c.z;
   t.nav = __float_as_uint(c.w);
@@ -49,29 +61,34 @@ __device__ __forceinline__ void load_track<float>(const TrackSoA& q, uint32_t i,
 }
 
 template <class R>
-__device__ __forceinline__ void store_track(const TrackSoA& q, uint32_t i, double x, double y, double z, R ux,
-                                            R uy, R uz, double E, unsigned long long id, uint32_t ev,
-                                            uint32_t step, uint32_t nav);
+__device__ __forceinline__ void store_track(char* q, uint32_t i, double x, double y, double z, R ux, R uy, R uz, double E,
+                                            unsigned long long id, uint32_t ev, uint32_t step, uint32_t nav);
 template <>
-__device__ __forceinline__ void store_track<double>(const TrackSoA& q, uint32_t i, double x, double y, double z,
-                                                    double ux, double uy, double uz, double E, unsigned long long id,
-                                                    uint32_t ev, uint32_t step, uint32_t nav) {
-  q.x[i] = x; q.y[i] = y; q.z[i] = z;
-  q.ux[i] = ux; q.uy[i] = uy; q.uz[i] = uz;
-  q.E[i] = E;
-  q.id[i] = id;
-  q.ev[i] = ev;
-  q.step[i] = step;
-  q.nav[i] = nav;
+__device__ __forceinline__ void store_track<double>(char* q, uint32_t i, double x, double y, double z, double ux, double uy,
+                                                    double uz, double E, unsigned long long id, uint32_t ev, uint32_t step,
+                                                    uint32_t nav) {
+  using L = Tile<double>;
+  char* a = q + (size_t)(i >> 5) * L::kBytes;
+  double* d = (double*)a + (i & 31u);
+  uint32_t* w = (uint32_t*)(a + L::kEv) + (i & 31u);
+  d[L::kX / 8] = x; d[L::kY / 8] = y; d[L::kZ / 8] = z;
+  d[L::kUX / 8] = ux; d[L::kUY / 8] = uy; d[L::kUZ / 8] = uz;
+  d[L::kE / 8] = E;
+  ((unsigned long long*)d)[L::kId / 8] = id;
+  w[0] = ev;
+  w[(L::kStep - L::kEv) / 4] = step;
+  w[(L::kNav - L::kEv) / 4] = nav;
 }
 template <>
-__device__ __forceinline__ void store_track<float>(const TrackSoA& q, uint32_t i, double x, double y, double z,
-                                                   float ux, float uy, float uz, double E, unsigned long long id,
-                                                   uint32_t ev, uint32_t step, uint32_t nav) {
-  q.xy[i] = make_double2(x, y);
-  q.zE[i] = make_double2(z, E);
-  q.un[i] = make_float4(ux, uy, uz, __uint_as_float(nav));
-  q.meta[i] = make_uint4((uint32_t)id, (uint32_t)(id >> 32), ev, step);
+__device__ __forceinline__ void store_track<float>(char* q, uint32_t i, double x, double y, double z, float ux, float uy,
+                                                   float uz, double E, unsigned long long id, uint32_t ev, uint32_t step,
+                                                   uint32_t nav) {
+  using L = Tile<float>;
+  char* r = q + (size_t)(i >> 5) * L::kBytes + (i & 31u) * 16u;
+  *(double2*)(r + L::kXY) = make_double2(x, y);
+  *(double2*)(r + L::kZE) = make_double2(z, E);
+  *(float4*)(r + L::kUN) = make_float4(ux, uy, uz, __uint_as_float(nav));
+  *(uint4*)(r + L::kMeta) = make_uint4((uint32_t)id, (uint32_t)(id >> 32), ev, step);
 }
 
 // an outgoing particle (paper Sec. 4: the GPU region hands back the particles that leave it)
@@ -359,7 +376,7 @@ __device__ __forceinline__ void emit(const Params& P, int p, int cw, const Trk<R
     if (alive) {
       const uint32_t d = bk + __popc(bs & lt);
       if (d < P.cap) {
-        store_track<R>(P.qd[3 * (p ^ 1) + S], d, t.x, t.y, t.z, t.u[0], t.u[1], t.u[2], t.E, t.id, t.ev, t.step, t.nav);
+        store_track<R>(track_queue(P, p ^ 1, S), d, t.x, t.y, t.z, t.u[0], t.u[1], t.u[2], t.E, t.id, t.ev, t.step, t.nav);
       } else {
         atomicAdd(&P.ctrl->overflow, 1ull);
         atomicAdd(P.evt.killed + t.ev, t.E + (S == 2 ? 2.0 * kMe : 0.0));
@@ -382,13 +399,12 @@ __device__ __forceinline__ void emit(const Params& P, int p, int cw, const Trk<R
     wbase[k] = __shfl_sync(0xFFFFFFFFu, bk, 0);
     ncreated[k] += __popc(b1[k]) + __popc(b2[k]);
   }
-  const TrackSoA* nq = P.qd + 3 * (p ^ 1);
   // pick entry k of a 3-array without dynamic indexing (which would place it in local memory)
   auto pick = [](const uint32_t* a, int k) { return k == 0 ? a[0] : (k == 1 ? a[1] : a[2]); };
   if (alive) {
     const uint32_t d = wbase[S] + __popc(b0[S] & lt);
     if (d < P.cap) {
-      store_track<R>(nq[S], d, t.x, t.y, t.z, t.u[0], t.u[1], t.u[2], t.E, t.id, t.ev, t.step, t.nav);
+      store_track<R>(track_queue(P, p ^ 1, S), d, t.x, t.y, t.z, t.u[0], t.u[1], t.u[2], t.E, t.id, t.ev, t.step, t.nav);
     } else {
       atomicAdd(&P.ctrl->overflow, 1ull);
       atomicAdd(P.evt.killed + t.ev, t.E + (S == 2 ? 2.0 * kMe : 0.0));
@@ -404,7 +420,7 @@ __device__ __forceinline__ void emit(const Params& P, int p, int cw, const Trk<R
     const uint32_t d = pick(wbase, sk) + before + mine;
     if (d < P.cap) {
       const unsigned long long cid = child_id(P.seed, __ldg(P.evt.key + t.ev), t.id, pstep, (uint32_t)k);
-      store_track<R>(nq[sk], d, t.x, t.y, t.z, sec.d[k][0], sec.d[k][1], sec.d[k][2], sec.E[k], cid, t.ev, 0u,
+      store_track<R>(track_queue(P, p ^ 1, sk), d, t.x, t.y, t.z, sec.d[k][0], sec.d[k][1], sec.d[k][2], sec.E[k], cid, t.ev, 0u,
                      vnav);
     } else {
       atomicAdd(&P.ctrl->overflow, 1ull);
@@ -431,20 +447,14 @@ template <class R> struct WarpRing {
 };
 
 // Tiles go to a warp in a fixed stride, so its next tile is known while it steps this one:
-// 16 lanes each ask L2 for one of the next tile's 16 lines of track records (4 arrays x 512
-// bytes), so that the tile's loads find them there instead of in DRAM (+0.9 % on the 10 GeV
-// showers; two tiles ahead gained less). FP32 form: the FP64 form is bound by its FP64 pipe.
-template <class R, int S>
-__device__ __forceinline__ void prefetch_tile(const Params& P, int p, uint32_t tile, uint32_t n, uint32_t lane) {
+// 16 lanes each ask L2 for one of the next tile's 16 lines, so that the tile's loads find
+// them there instead of in DRAM (+0.9 % on the 10 GeV showers; two tiles ahead gained less).
+// FP32 form: the FP64 form is bound by its FP64 pipe.
+template <class R>
+__device__ __forceinline__ void prefetch_tile(const char* q, uint32_t tile, uint32_t lane) {
   if constexpr (sizeof(R) == 4) {
-    const uint32_t e0 = (tile << 5) + ((lane & 3u) << 3);  // first of the 8 records in this lane's line
-    if (lane < 16u && e0 < n) {
-      const TrackSoA& q = P.qd[3 * p + S];
-      const uint32_t a = lane >> 2;
-      const char* b = a == 0 ? (const char*)q.xy
-                             : (a == 1 ? (const char*)q.zE : (a == 2 ? (const char*)q.un : (const char*)q.meta));
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(b + (size_t)e0 * 16));
-    }
+    if (lane < 16u)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(q + (size_t)tile * Tile<R>::kBytes + lane * 128u));
   }
 }
 
@@ -474,8 +484,9 @@ __device__ __forceinline__ void run_tiles(const Params& P, int p, int cw, uint32
     if (phase_a) {
       const uint32_t i = (tile << 5) + lane;
       const bool active = i < n;
-      if (active) load_track<R>(P.qd[3 * p + S], i, t);
-      if (tile + stride < tiles) prefetch_tile<R, S>(P, p, tile + stride, n, lane);
+      const char* q = track_queue(P, p, S);
+      if (active) load_track<R>(q, tile, lane, t);
+      if (tile + stride < tiles) prefetch_tile<R>(q, tile + stride, lane);
       if (active) outcome = step_transport<R, S, V>(P, t, sec, dep, bin, pstep, proc);
       nsteps[S] += active ? 1u : 0u;  // per lane; reduced over the warp at the end
     } else if (lane < c) {
