@@ -148,17 +148,15 @@ struct adept_ctx {
   int fgrid = 0, fminb = 0;  // fused generation kernel
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // one per status buffer (own timing events)
   int graph_gens = 0;
-  // tail chunks (one per status buffer): a conditional while node runs one generation per
-  // iteration until the queues are empty, so the end of a transport launches no empty
-  // generations; chosen once the live tracks at the last status fall below kTailTracks
-  cudaGraphExec_t tgraph[2] = {nullptr, nullptr};
+  // tail chunks: one kernel runs the generations of a small population until the queues are
+  // empty (tail.cuh), while fewer than tail_tracks tracks are live
+  uint32_t tail_tracks = 0;       // 0: never
+  int tail_blocks = 0;
   bool tail[2] = {false, false};  // the chunk queued in buffer b is a tail chunk
   uint64_t last_live = 0;         // live tracks at the end of the last chunk read back
-  uint64_t peak_live = 0;         // most live tracks seen since the queues were last empty
   // estimated peak tracks (tracks_per_MeV x energy, plus the primaries) of the requests
   // admitted so far; its value when chunk b was launched; and the value behind last_live
   uint64_t admit_est = 0, admit_mark[2] = {0, 0}, admit_seen = 0;
-  cudaStream_t bstream = nullptr; // captures the tail chunks' loop body
   std::vector<cudaEvent_t> ev;  // 4 per generation when timing: start, after e-, after e+, after gamma
   cudaStream_t side[2] = {nullptr, nullptr};     // the e+ and gamma kernels run on these
   cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
@@ -424,7 +422,11 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   P.chord_iter = o.field_max_iterations;
   P.delta_chord = o.delta_chord_mm;
   P.delta_int = o.delta_intersection_mm;
-  P.tail_exit = o.tail_tracks > 0 ? (uint32_t)std::min<uint64_t>(4ull * (uint64_t)o.tail_tracks, 0xFFFFFFFFull) : 0u;
+  // no tail kernel with the optional physics: its multiple scattering rounds differently in
+  // another kernel (FP32), and a history must not depend on which kernel steps it
+  if (o.tail_tracks > 0 && !o.physics)
+    c->tail_tracks = std::min<uint32_t>((uint32_t)o.tail_tracks, o.precision ? kTailTracks : kTailTracksFp64);
+  P.tail_exit = 2 * c->tail_tracks;
   c->steplen = steplen;
   // device state
   adept_ctx* c_ = cp;
@@ -463,7 +465,6 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
     }
     CK(cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming));
     CK(cudaStreamCreateWithFlags(&c->tstream, cudaStreamNonBlocking));
-    CK(cudaStreamCreateWithFlags(&c->bstream, cudaStreamNonBlocking));
     for (int j = 0; j < 3; ++j) CK(cudaEventCreateWithFlags(&c->kdone[j], cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&c->tjoin, cudaEventDisableTiming));
     CK(cudaStreamSynchronize(c->stream));
@@ -479,6 +480,7 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
       int bps = transport_max_blocks_per_sm(o.precision, sp, c->minb[sp], o.block_size, transport_variant(P));
       c->grid[sp] = sms * (bps < 1 ? 1 : bps);
     }
+    if (c->tail_tracks) c->tail_blocks = tail_blocks(P, o.precision, o.fused != 0);
     if (o.fused) {
       int mb = o.blocks_per_sm > 0 ? o.blocks_per_sm : (o.precision ? 2 : 1);
       c->fminb = std::min(4, mb);
@@ -752,79 +754,6 @@ static cudaError_t enqueue_generations(adept_ctx* c, int gens, int b, bool captu
   return e;
 }
 
-// Below adept_options.tail_tracks live tracks a generation is dominated by its launch, and
-// a tail chunk trades the programmatic launch between generations (about 5 us a generation
-// on GB300) for stopping exactly when the last track dies (a fixed chunk runs to its end, and
-// one more is queued behind it: at the end of a transport the rest of the one and all of the
-// other run on empty queues). So tail chunks are
-// kept for the decay at the end: fewer live tracks than tail_tracks and than a kTailDecay-th
-// of the peak since the queues were last empty. A tail chunk runs at most
-// graph_generations generations, like a fixed one, so the status is read as often.
-constexpr uint64_t kTailDecay = 8;
-
-// A tail chunk: open (condition = live tracks) -> while (condition) { one generation (the
-// three species kernels, or the fused kernel) -> step (++tail_k, condition = live tracks,
-// fewer than 4 tail_tracks, and tail_k < graph_generations) } -> end of chunk with the count
-// the loop left. No timing records (event nodes are not allowed in a conditional body).
-static int capture_tail_graph(adept_ctx* c, int b) {
-  cudaGraph_t g = nullptr;
-  cudaGraphConditionalHandle h;
-  cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) return fail(c, ADEPT_ECUDA, "tail capture: %s", cudaGetErrorString(e));
-  cudaStreamCaptureStatus cs;
-  const cudaGraphNode_t* deps = nullptr;
-  size_t ndeps = 0;
-  e = launch_open_chunk(c->P, b, c->stream);
-  if (e == cudaSuccess) e = cudaStreamGetCaptureInfo(c->stream, &cs, nullptr, &g, nullptr, nullptr, nullptr);
-  if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault);
-  if (e == cudaSuccess) e = launch_tail_open(c->P, h, c->stream);
-  if (e == cudaSuccess) e = cudaStreamGetCaptureInfo(c->stream, &cs, nullptr, &g, &deps, nullptr, &ndeps);
-  cudaGraphNode_t loop = nullptr;
-  cudaGraph_t body = nullptr;
-  if (e == cudaSuccess) {
-    cudaGraphNodeParams cp = {};
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = h;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    e = cudaGraphAddNode(&loop, g, deps, nullptr, ndeps, &cp);
-    if (e == cudaSuccess) body = cp.conditional.phGraph_out[0];
-  }
-  if (e == cudaSuccess) e = cudaStreamUpdateCaptureDependencies(c->stream, &loop, nullptr, 1, cudaStreamSetCaptureDependencies);
-  // the loop body: one generation, captured on a stream of its own
-  if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(c->bstream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
-  if (e == cudaSuccess) {
-    cudaStream_t s0 = c->bstream;
-    if (c->opt.fused) {
-      e = launch_fused_generation(c->P, kGkDevice, c->opt.precision, c->fminb, c->fgrid, c->block, false, s0);
-    } else {
-      e = cudaEventRecord(c->fork, s0);
-      for (int j = 0; j < 2 && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(c->side[j], c->fork, 0);
-      cudaStream_t st[3] = {c->side[1], s0, c->side[0]};  // gamma, e-, e+
-      for (int sp : {0, 2, 1})
-        if (e == cudaSuccess) e = launch_transport(c->P, kGkDevice, c->opt.precision, sp, c->minb[sp], c->grid[sp], c->block, false, st[sp]);
-      for (int j = 0; j < 2 && e == cudaSuccess; ++j) e = cudaEventRecord(c->join[j], c->side[j]);
-      for (int j = 0; j < 2 && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(s0, c->join[j], 0);
-    }
-    if (e == cudaSuccess) e = launch_tail_step(c->P, h, (uint32_t)c->opt.graph_generations, s0);
-    cudaGraph_t bg = nullptr;
-    const cudaError_t e3 = cudaStreamEndCapture(s0, &bg);
-    if (e == cudaSuccess) e = e3;
-  }
-  if (e == cudaSuccess) e = launch_finish(c->P, b, kGkDevice, c->stream);
-  cudaGraph_t out = nullptr;
-  const cudaError_t e2 = cudaStreamEndCapture(c->stream, &out);
-  if (e != cudaSuccess) {
-    if (out) cudaGraphDestroy(out);
-    return fail(c, ADEPT_ECUDA, "tail graph capture: %s", cudaGetErrorString(e));
-  }
-  if (e2 != cudaSuccess) return fail(c, ADEPT_ECUDA, "tail graph capture end: %s", cudaGetErrorString(e2));
-  e = cudaGraphInstantiate(&c->tgraph[b], out, 0);
-  cudaGraphDestroy(out);
-  if (e != cudaSuccess) return fail(c, ADEPT_ECUDA, "tail graph instantiate: %s", cudaGetErrorString(e));
-  return ADEPT_OK;
-}
-
 static int capture_graph(adept_ctx* c, int gens, int b) {
   cudaGraph_t g;
   CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
@@ -851,16 +780,13 @@ static int launch_chunk(adept_ctx* c, int b) {
     if (rc) return rc;
   }
   const uint64_t live = c->last_live + (c->admit_est - c->admit_seen);
-  c->tail[b] = G > 0 && c->opt.tail_tracks > 0 && live < (uint64_t)c->opt.tail_tracks &&
-               live * kTailDecay < c->peak_live;
+  c->tail[b] = G > 0 && live < (uint64_t)c->tail_tracks;
   c->admit_mark[b] = c->admit_est;
   if (c->tail[b]) {
-    if (!c->tgraph[b]) {
-      int rc = capture_tail_graph(c, b);
-      if (rc) return rc;
-    }
-    CK(cudaGraphLaunch(c->tgraph[b], c->stream));
-    c->stats.launches += 5;  // chunk open, loop open, end of chunk, mark, finish; the loop's kernels once read back
+    CK(launch_open_chunk(c->P, b, c->stream));
+    CK(launch_tail(c->P, c->opt.precision, c->opt.fused != 0, c->tail_blocks, (uint32_t)gens, c->stream));
+    CK(launch_finish(c->P, b, kGkDevice, c->stream));
+    c->stats.launches += 5;  // chunk open, tail, end of chunk, mark, finish
   } else if (G > 0) {
     if (!c->graph[b]) {
       int rc = capture_graph(c, G, b);
@@ -880,11 +806,7 @@ static int launch_chunk(adept_ctx* c, int b) {
 // Wait for chunk b and account its timing events.
 static int wait_chunk(adept_ctx* c, int b) {
   CK(cudaEventSynchronize(c->status_ev[b]));
-  if (c->tail[b]) {  // the loop's generations: the species kernels (or the fused one) and a step kernel
-    c->stats.launches += (uint64_t)c->h_ctrl[b]->tail_k * ((c->opt.fused ? 1 : 3) + 1);
-    return ADEPT_OK;
-  }
-  if (timing(c)) {
+  if (timing(c) && !c->tail[b]) {  // tail chunks are not timed
     const int G = c->opt.graph_generations;
     const int gens = G > 0 ? G : 1;
     const cudaEvent_t* ev = c->ev.data() + 4 * gens * b;
@@ -1111,7 +1033,6 @@ extern "C" int adept_transport(adept_ctx* c, uint64_t timeout_us) {
     const uint32_t live = h.count[h.gen % 3][0].n + h.count[h.gen % 3][1].n + h.count[h.gen % 3][2].n;
     c->last_live = live;
     c->admit_seen = c->admit_mark[b];
-    c->peak_live = live ? std::max<uint64_t>(c->peak_live, live) : 0;
     // While tracks are live and no request waits for admission, relaunch buffer b at once, so
     // that the host's processing of this status (outgoing particles, finished events) overlaps
     // the next chunk instead of delaying the launch of the one after it: on the 10 GeV showers
@@ -1536,7 +1457,6 @@ extern "C" void adept_destroy(adept_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   for (int b = 0; b < 2; ++b) {
     if (c->graph[b]) cudaGraphExecDestroy(c->graph[b]);
-    if (c->tgraph[b]) cudaGraphExecDestroy(c->tgraph[b]);
   }
   for (auto e : c->ev) cudaEventDestroy(e);
   for (int j = 0; j < 2; ++j) {
@@ -1546,7 +1466,6 @@ extern "C" void adept_destroy(adept_ctx* c) {
   if (c->submit_stream) { cudaStreamSynchronize(c->submit_stream); cudaStreamDestroy(c->submit_stream); }
   if (c->fork) cudaEventDestroy(c->fork);
   if (c->tstream) { cudaStreamSynchronize(c->tstream); cudaStreamDestroy(c->tstream); }
-  if (c->bstream) cudaStreamDestroy(c->bstream);
   for (int j = 0; j < 3; ++j)
     if (c->kdone[j]) cudaEventDestroy(c->kdone[j]);
   if (c->tjoin) cudaEventDestroy(c->tjoin);

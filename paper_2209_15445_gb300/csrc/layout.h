@@ -97,7 +97,7 @@ struct Ctrl {
   uint32_t done_count[2];     // events found finished by the finish pass of a chunk (per buffer)
   uint32_t log_n;             // rows written to the generation log
   uint32_t error;             // first device-detected error code (0 = none)
-  uint32_t tail_k;            // generations a tail chunk has run so far (see kGkDevice)
+  uint32_t tail_k;            // generations the last tail chunk ran (see kGkDevice)
   uint32_t finish_ticket;     // blocks of the finish pass that have ended (the last one resets it)
   uint32_t pad[2];
   unsigned long long steps[3];
@@ -182,10 +182,20 @@ cudaError_t launch_build_tables(const Params& P, const double* mat_in, int n_mat
                                 float2* g32, float2* e32, float2* p32, double* re64, double* rp64,
                                 float* re32, float* rp32, uint16_t* const range_index[4], double* Tc, double* kc,
                                 cudaStream_t st);
-// A tail chunk runs its generations as the body of a conditional (while) graph node, one
-// generation per iteration, until the queues are empty or a cap is reached; its kernels are
-// launched with gk = kGkDevice and read their place in the chunk from Ctrl::tail_k.
+// A tail chunk: up to max_gens generations in one launch (tail.cuh), fewer if the queues run
+// empty or P.tail_exit tracks are live; the count is left in Ctrl::tail_k, which the end of the
+// chunk reads when its gens is kGkDevice.
 constexpr uint32_t kGkDevice = 0xFFFFFFFFu;
+// It takes over below kTailTracks live tracks and ends at twice as many. Where the lines lie
+// (ms, by kTailTracks): 10 showers of 10 GeV 2.20 (4096), 2.13 (8192), 2.04 (16384), 2.38 with
+// fixed chunks; 100 showers 2.84, 2.84, 2.75, 3.15; a round of 16 serving requests 4.55, 4.56,
+// 4.62, 5.1. FP64, whose generations want more SMs: 10 showers 6.8 (512 to 2048), 8.4 (8192).
+constexpr uint32_t kTailTracks = 12288, kTailTracksFp64 = 2048;
+cudaError_t launch_tail(const Params& P, int precision, bool fused, int blocks, uint32_t max_gens, cudaStream_t st);
+// blocks of its cluster (one a species in turn): 16, or 8 where no cluster of 16 can be resident
+int tail_blocks(const Params& P, int precision, bool fused);
+// its kernels with chords, and with the step-length histogram
+const void* tail_variant_fn(int precision, int variant);
 // generation gen + gk of one species (gk: its place in the chunk; the three species of a
 // generation may run concurrently). pdl: launch with a programmatic dependency on the
 // stream's preceding kernels (the previous generation's), see grid_dependency_wait.
@@ -202,10 +212,6 @@ cudaError_t launch_open_chunk(const Params& P, int b, cudaStream_t st);
 // Ctrl::tail_k): log the last one, advance gen, find finished events, and write the status
 // and the done list to the host's copy of buffer b
 cudaError_t launch_finish(const Params& P, int buffer, uint32_t gens, cudaStream_t st);
-// tail chunks: before the loop, tail_k = 0 and the condition = live tracks in the queues;
-// after each generation, ++tail_k and the condition = live tracks and tail_k < max_gens
-cudaError_t launch_tail_open(const Params& P, cudaGraphConditionalHandle h, cudaStream_t st);
-cudaError_t launch_tail_step(const Params& P, cudaGraphConditionalHandle h, uint32_t max_gens, cudaStream_t st);
 cudaError_t launch_probe_philox(const uint32_t* ctr, int n, uint32_t k0, uint32_t k1, uint32_t* out,
                                 cudaStream_t st);
 cudaError_t launch_probe_interp(const Params& P, int s, int t, int m, int prec, const double* E, int n,

@@ -1,0 +1,55 @@
+// The tail kernels of the default steps, without and with the helix in a field (variants 0 and
+// 8 of step_transport), for contexts with species kernels and, with the rounding of that form,
+// with the fused one, and the launch of every variant's.
+#include <cuda_runtime.h>
+
+#include "layout.h"
+#include "tail.cuh"
+
+namespace adept {
+
+template <class R>
+static const void* tail_fn(int variant, bool fused) {
+  if (fused) return (variant & 8) ? (const void*)k_tail<R, 0, 24> : (const void*)k_tail<R, 0, 16>;
+  if (variant & 5) return tail_variant_fn(sizeof(R) == 4, variant);
+  return (variant & 8) ? (const void*)k_tail<R, 0, 8> : (const void*)k_tail<R, 0, 0>;
+}
+
+static void tail_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int blocks, cudaStream_t st) {
+  cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = blocks;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+}
+
+static const void* tail_fn(const Params& P, int precision, bool fused) {
+  return precision ? tail_fn<float>(transport_variant(P), fused) : tail_fn<double>(transport_variant(P), fused);
+}
+
+int tail_blocks(const Params& P, int precision, bool fused) {
+  const void* fn = tail_fn(P, precision, fused);
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  tail_config(cfg, at, 16, nullptr);
+  int n = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0)
+    return 16;
+  (void)cudaGetLastError();
+  return 8;
+}
+
+cudaError_t launch_tail(const Params& P, int precision, bool fused, int blocks, uint32_t max_gens, cudaStream_t st) {
+  void* args[] = {const_cast<Params*>(&P), &max_gens};
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  tail_config(cfg, at, blocks, st);
+  return cudaLaunchKernelExC(&cfg, tail_fn(P, precision, fused), args);
+}
+
+}  // namespace adept

@@ -28,30 +28,32 @@ __device__ __forceinline__ uint32_t track_event(const Params& P, const char* q, 
                  : *(const uint32_t*)(q + (size_t)(i >> 5) * Tile<double>::kBytes + Tile<double>::kEv + (i & 31u) * 4u);
 }
 
-// Queue loads are streaming (ld.global.cs): each slot is read once per generation.
-template <class R>
-__device__ __forceinline__ void load_track(const char* q, uint32_t tile, uint32_t lane, Trk<R>& t);
-template <>
-__device__ __forceinline__ void load_track<double>(const char* q, uint32_t tile, uint32_t lane, Trk<double>& t) {
+// Queue loads are streaming (ld.global.cs): each slot is read once per generation. The tail
+// kernel (L2 = true) reads in one generation what other SMs wrote in the one before, and goes
+// to L2 (ld.global.cg; everywhere it took 33.1 instead of 32.7 ms on 10,000 10 GeV showers).
+template <bool L2, class T> __device__ __forceinline__ T load_stream(const T* p) { return L2 ? __ldcg(p) : __ldcs(p); }
+template <bool L2>
+__device__ __forceinline__ void load_track(const char* q, uint32_t tile, uint32_t lane, Trk<double>& t) {
   using L = Tile<double>;
   const char* a = q + (size_t)tile * L::kBytes;
   const double* d = (const double*)a + lane;
   const uint32_t* w = (const uint32_t*)(a + L::kEv) + lane;
-  t.x = __ldcs(d + L::kX / 8); t.y = __ldcs(d + L::kY / 8); t.z = __ldcs(d + L::kZ / 8);
-  t.u[0] = __ldcs(d + L::kUX / 8); t.u[1] = __ldcs(d + L::kUY / 8); t.u[2] = __ldcs(d + L::kUZ / 8);
-  t.E = __ldcs(d + L::kE / 8);
-  t.id = __ldcs((const unsigned long long*)d + L::kId / 8);
-  t.ev = __ldcs(w);
-  t.step = __ldcs(w + (L::kStep - L::kEv) / 4);
-  t.nav = __ldcs(w + (L::kNav - L::kEv) / 4);
+  t.x = load_stream<L2>(d + L::kX / 8); t.y = load_stream<L2>(d + L::kY / 8); t.z = load_stream<L2>(d + L::kZ / 8);
+  t.u[0] = load_stream<L2>(d + L::kUX / 8); t.u[1] = load_stream<L2>(d + L::kUY / 8);
+  t.u[2] = load_stream<L2>(d + L::kUZ / 8);
+  t.E = load_stream<L2>(d + L::kE / 8);
+  t.id = load_stream<L2>((const unsigned long long*)d + L::kId / 8);
+  t.ev = load_stream<L2>(w);
+  t.step = load_stream<L2>(w + (L::kStep - L::kEv) / 4);
+  t.nav = load_stream<L2>(w + (L::kNav - L::kEv) / 4);
 }
-template <>
-__device__ __forceinline__ void load_track<float>(const char* q, uint32_t tile, uint32_t lane, Trk<float>& t) {
+template <bool L2>
+__device__ __forceinline__ void load_track(const char* q, uint32_t tile, uint32_t lane, Trk<float>& t) {
   using L = Tile<float>;
   const char* r = q + (size_t)tile * L::kBytes + lane * 16u;
-  const double2 a = __ldcs((const double2*)(r + L::kXY)), b = __ldcs((const double2*)(r + L::kZE));
-  const float4 c = __ldcs((const float4*)(r + L::kUN));
-  const uint4 d = __ldcs((const uint4*)(r + L::kMeta));
+  const double2 a = load_stream<L2>((const double2*)(r + L::kXY)), b = load_stream<L2>((const double2*)(r + L::kZE));
+  const float4 c = load_stream<L2>((const float4*)(r + L::kUN));
+  const uint4 d = load_stream<L2>((const uint4*)(r + L::kMeta));
   t.x = a.x; t.y = a.y; t.z = b.x; t.E = b.y;
   t.u[0] = c.x; t.u[1] = c.y; t.u[2] = c.z;
   t.nav = __float_as_uint(c.w);
@@ -140,7 +142,8 @@ enum Outcome { kDead = 0, kAlive = 1, kInteract = 2 };
 // fluctuations (P.physics), bit 2 the validation histogram of step lengths (P.steplen;
 // its never-taken branch cost the default kernels 1.6 %), bit 3 the helix of a charged
 // track in the uniform field (P.field_T != 0; without it a track moves straight, and the
-// kernels for the field-free calorimeters carry no helix code: +1.5 %).
+// kernels for the field-free calorimeters carry no helix code: +1.5 %), bit 4 the rounding of
+// the one-kernel-per-generation form (see transverse2).
 template <class R, int S, int V = 0>
 __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>& sec, double& dep, int& dep_bin,
                                               uint32_t& pstep, int& proc) {
@@ -218,6 +221,9 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
   // S5/S6: distance to the boundary along the straight line or helix
   int next;
   const bool field = (V & 8) != 0 && (q != 0) && (P.field_T != 0.0);
+  // the rounding of the navigation (see transverse2): written out but in the optional-physics
+  // kernels, which have no tail kernel beside them (chords have their own)
+  constexpr int F = (V & 2) != 0 ? 0 : (S != 0 && ((V & 16) != 0 || sizeof(R) == 8) ? 2 : 1);
   bool boundary;
   R s;
   if constexpr (CH) {
@@ -230,12 +236,12 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
     boundary = rc == 1;
     s = sd;
   } else {
-    const R s_geom = field ? helix_distance<R>(P.geo, P.field_T, t.E, q, t.x, t.y, t.z, t.u, vol, &next)
-                           : straight_distance<R>(P.geo, t.x, t.y, t.z, t.u, vol, &next);
+    const R s_geom = field ? helix_distance<R, F>(P.geo, P.field_T, t.E, q, t.x, t.y, t.z, t.u, vol, &next)
+                           : straight_distance<R, F>(P.geo, t.x, t.y, t.z, t.u, vol, &next);
     boundary = s_geom <= s_phys;
     s = boundary ? s_geom : s_phys;
     if (field) {
-      helix_move<R>(P.field_T, t.E, q, s, &t.x, &t.y, &t.z, t.u);
+      helix_move<R, F>(P.field_T, t.E, q, s, &t.x, &t.y, &t.z, t.u);
     } else {
       t.x += to_d<R>(s * t.u[0]);
       t.y += to_d<R>(s * t.u[1]);
@@ -464,7 +470,7 @@ __device__ __forceinline__ void prefetch_tile(const char* q, uint32_t tile, uint
 // warp of up to 32 queued interactions. Both share the scoring and the appends, so every
 // part of the step is inlined once per kernel (smaller code: fewer instruction-cache
 // misses).
-template <class R, int S, int V = 0>
+template <class R, int S, int V = 0, bool L2 = false>
 __device__ __forceinline__ void run_tiles(const Params& P, int p, int cw, uint32_t tile, uint32_t tiles, uint32_t stride,
                                           uint32_t n, WarpRing<R>& ring, uint32_t* nsteps, uint32_t* ncreated) {
   const uint32_t lane = threadIdx.x & 31;
@@ -485,7 +491,7 @@ __device__ __forceinline__ void run_tiles(const Params& P, int p, int cw, uint32
       const uint32_t i = (tile << 5) + lane;
       const bool active = i < n;
       const char* q = track_queue(P, p, S);
-      if (active) load_track<R>(q, tile, lane, t);
+      if (active) load_track<L2>(q, tile, lane, t);
       if (tile + stride < tiles) prefetch_tile<R>(q, tile + stride, lane);
       if (active) outcome = step_transport<R, S, V>(P, t, sec, dep, bin, pstep, proc);
       nsteps[S] += active ? 1u : 0u;  // per lane; reduced over the warp at the end
@@ -521,6 +527,9 @@ __device__ __forceinline__ void run_tiles(const Params& P, int p, int cw, uint32
     __syncwarp();
   }
 }
+
+// A warp's first tile in a grid that takes the tiles in a stride of all its warps.
+__device__ __forceinline__ uint32_t first_tile() { return blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); }
 
 // Programmatic dependent launch between generations: a generation's kernels may be
 // launched (and their blocks made resident) as soon as every block of the previous
@@ -561,7 +570,6 @@ __global__ void __launch_bounds__(256, MINB) k_transport(Params P, uint32_t gk) 
   __shared__ WarpRing<R> rings[8];
   grid_dependency_wait();
   allow_dependent_launch();
-  if (gk == kGkDevice) gk = __ldcg(&P.ctrl->tail_k);  // a generation of a tail chunk
   const uint32_t gen = __ldcg(&P.ctrl->gen) + gk;
   const int p = gen & 1;
   if (threadIdx.x == 0) { s_steps = 0; s_created[0] = s_created[1] = s_created[2] = 0; }
@@ -577,7 +585,7 @@ __global__ void __launch_bounds__(256, MINB) k_transport(Params P, uint32_t gk) 
   // lane, reduced over the warp at the end (a ballot per pass measured 1.2 % slower), and
   // secondaries per warp
   uint32_t nsteps[3] = {0, 0, 0}, ncreated[3] = {0, 0, 0};
-  run_tiles<R, S, V>(P, p, (gen + 1) % 3, blockIdx.x * wpb + (threadIdx.x >> 5), tiles, gridDim.x * wpb, n, ring,
+  run_tiles<R, S, V>(P, p, (gen + 1) % 3, first_tile(), tiles, gridDim.x * wpb, n, ring,
                      nsteps, ncreated);
   const uint32_t wsteps = __reduce_add_sync(0xFFFFFFFFu, nsteps[S]);
   if ((threadIdx.x & 31) == 0) {
