@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(256, MINB) k_fused_generation(Params P, uint32
   const uint32_t n2 = min(__ldcg(&P.ctrl->count[cr][2].n), P.cap);
   const uint32_t T0 = (n0 + 31) >> 5, T1 = (n1 + 31) >> 5, T2 = (n2 + 31) >> 5;
   uint32_t nsteps[3] = {0, 0, 0}, ncreated[3] = {0, 0, 0};  // this generation: steps per lane, secondaries per warp
-  uint32_t first = first_tile();
+  uint32_t first = first_tile<R, V>();
   run_tiles<R, 0, V | 16>(P, p, cw, first, T0, nwarps, n0, ring, nsteps, ncreated);
   first = next_first(first, T0, nwarps);
   run_tiles<R, 1, V | 16>(P, p, cw, first, T1, nwarps, n1, ring, nsteps, ncreated);
