@@ -407,6 +407,7 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   P.geo.kind = c->kind; P.geo.n_vol = c->n_vol; P.geo.n_bins = c->n_bins;
   P.geo.half_xy = geometry->transverse_half_mm; P.geo.half_z = geometry->half_length_mm;
   P.geo.safe_xy = (float)(geometry->transverse_half_mm * 0.9999 - 2.0);
+  P.geo.safe_z = (float)(geometry->half_length_mm * 0.9999 - 2.0);
   P.geo.bnd = bnd; P.geo.vol_mat = vm; P.geo.vol_bin = vb;
   P.mat = c->mat_dev;
   P.tab = TableView{c->g64, c->e64, c->p64, c->g32, c->e32, c->p32, c->re64, c->rp64, c->re32, c->rp32,

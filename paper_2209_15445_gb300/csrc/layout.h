@@ -21,7 +21,7 @@ struct GeoView {
   int n_vol;
   int n_bins;
   double half_xy, half_z;
-  float safe_xy;         // slab: the wall half width less 1e-4 of it and 2 mm (inside_walls)
+  float safe_xy, safe_z; // slab: the wall half width less 1e-4 of it and 2 mm (inside_walls); tubes: the half length
   const double* bnd;     // slab: n_vol+1 planes; tubes: n_vol radii
   const int* vol_mat;    // material index or -1 (vacuum)
   const int* vol_bin;    // scoring bin or -1

@@ -57,3 +57,36 @@ def test_nearest_plane_or_wall(prec):
     up = np.where((step >= 0) & (step < len(planes) - 1), step, -1)
     clear = finite & (np.abs(sz - sw.min(axis=1)) > 2 * tol)
     np.testing.assert_array_equal(nxt[clear], np.where(sz < sw.min(axis=1), up, -1)[clear])
+
+
+@pytest.mark.parametrize("charge,tol", [(0, 1e-11), (-1, 1e-9)])
+def test_tubes_near_and_far_from_the_end_caps(charge, tol):
+    """FP64 tube distances, straight and along a helix, around the test that spares the distance
+    to the end caps, against the oracle (tolerances of the other tube distances)."""
+    need_gpu()
+    import oracle
+    from paper_2209_15445_gb300 import adept as A
+    rng = np.random.default_rng(6)
+    geom = W.barrel_calorimeter()
+    orc = oracle.Oracle(geom, field_T=3.8)
+    n = 4000
+    r, phi = rng.uniform(10.0, 1790.0, n), rng.uniform(0.0, 2 * np.pi, n)
+    cap = 3000.0 - rng.choice([1e-9, 0.01, 1.0, 2.0, 2.3, 2.4, 50.0, 1000.0], n)
+    z = np.where(rng.random(n) < 0.5, cap, -cap)
+    c = np.where(rng.random(n) < 0.3, rng.choice([0.0, 1.0, -1.0, 0.9999], n), rng.uniform(-1.0, 1.0, n))
+    f = rng.uniform(0.0, 2 * np.pi, n)
+    s = np.sqrt(1.0 - c * c)
+    pos = np.stack([r * np.cos(phi), r * np.sin(phi), z], 1)
+    d = np.stack([s * np.cos(f), s * np.sin(f), c], 1)
+    vol = np.array([orc.locate(p, u) for p, u in zip(pos, d)], np.int32)
+    T = np.exp(rng.uniform(np.log(0.05), np.log(5e3), n))
+    q = np.full(n, charge, np.int32)
+    tr = make(geom, precision=0, field_T=3.8)
+    rc, got, nxt = A.adept_probe_distance(tr.h, 0, pos, d, vol, T, q)
+    tr.close()
+    assert rc == 0
+    ref = [orc.helix_distance(t, charge, p, u, v) if charge else orc.distance(p, u, v) for p, u, v, t in zip(pos, d, vol, T)]
+    rs, rn = np.array([x[0] for x in ref]), np.array([x[1] for x in ref])
+    agree = np.abs(got - rs) <= tol * np.maximum(1.0, rs)
+    assert agree.mean() > 0.999
+    np.testing.assert_array_equal(nxt[agree], rn[agree])
