@@ -502,7 +502,7 @@ extern "C" int adept_build_tables(adept_ctx* c) {
   CK(launch_build_tables(c->P, c->mat_in, c->n_mat, c->range_cut, c->mat_dev, c->scratch, c->g64, c->e64, c->p64,
                          c->g32, c->e32, c->p32, c->re64, c->rp64, c->re32, c->rp32, c->xr, c->Tc, c->kc, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  c->stats.launches += 7;
+  c->stats.launches += 6;
   c->built = true;
   return ADEPT_OK;
 }

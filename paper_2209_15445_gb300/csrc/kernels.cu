@@ -4,91 +4,17 @@
 
 #include "device.cuh"
 #include "layout.h"
-#include "physics_init.cuh"
+#include "tables.cuh"
 #include "transport.cuh"
 
 namespace adept {
 
 // ======================================================================== table build
-// raw value rows in BuildScratch::vals
-enum { V_MUC, V_MUP, V_MUPH, V_SFULL, V_SE, V_IE, V_BE, V_SP, V_IP, V_BP, V_AP, V_RFULL, V_RE, V_RP, V_NROW };
-enum { B_RFULL, B_RE, B_RP };
-
-using init::bin_integral;
-using init::node_E;
-
-__global__ void k_materials(const double* in, int n, MatDev* out) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < n) init::setup_material(in + kMatRec * m, out + m);
-}
-
-__device__ inline double s_full(const MatDev& M, double T) {
-  return init::dedx_col(M, T, T, false) + init::dedx_rad(M, T, T);
-}
-__device__ inline double s_restr(const MatDev& M, double T, double Tc, double kc, bool pos) {
-  return init::dedx_col(M, T, Tc, pos) + init::dedx_rad(M, T, kc);
-}
-
-__global__ void k_gamma_full(const MatDev* mats, int n_mat, BuildScratch s) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n_mat * kNNode) return;
-  const int m = idx / kNNode, i = idx % kNNode;
-  const MatDev M = mats[m];
-  if (M.vacuum) return;
-  double* v = s.vals + (size_t)m * V_NROW * kNNode;
-  const double E = node_E(i);
-  v[V_MUC * kNNode + i] = init::mu_compton(M, E);
-  v[V_MUP * kNNode + i] = init::mu_pair(M, E);
-  v[V_MUPH * kNNode + i] = init::mu_photo(M, E);
-  v[V_SFULL * kNNode + i] = s_full(M, E);
-  if (i < kNNode - 1)
-    s.bins[((size_t)m * 3 + B_RFULL) * kNNode + i] = bin_integral(i, [&](double T) { return s_full(M, T); });
-}
-
-// production thresholds: e+- from the unrestricted range, gamma from 5 mean free paths
-__global__ void k_cuts(const MatDev* mats, int n_mat, double range_cut, BuildScratch s, double* Tc, double* kc) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= n_mat) return;
-  if (mats[m].vacuum) { Tc[m] = 0.0; kc[m] = 0.0; return; }
-  double* v = s.vals + (size_t)m * V_NROW * kNNode;
-  double* Rf = v + V_RFULL * kNNode;
-  init::prefix_range(v + V_SFULL * kNNode, s.bins + ((size_t)m * 3 + B_RFULL) * kNNode, Rf);
-  auto mu = [&](int i) { return v[V_MUC * kNNode + i] + v[V_MUP * kNNode + i] + v[V_MUPH * kNNode + i]; };
-  Tc[m] = init::clamp_cut(init::range_threshold(Rf, range_cut));
-  kc[m] = init::clamp_cut(init::gamma_threshold(mu, range_cut));
-}
-
-__global__ void k_charged(const MatDev* mats, int n_mat, BuildScratch s, const double* Tc, const double* kc) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n_mat * kNNode) return;
-  const int m = idx / kNNode, i = idx % kNNode;
-  const MatDev M = mats[m];
-  if (M.vacuum) return;
-  const double tc = Tc[m], kk = kc[m];
-  double* v = s.vals + (size_t)m * V_NROW * kNNode;
-  const double T = node_E(i);
-  v[V_SE * kNNode + i] = s_restr(M, T, tc, kk, false);
-  v[V_IE * kNNode + i] = init::lambda_ioni(M, T, tc, false);
-  v[V_BE * kNNode + i] = init::lambda_brem(M, T, kk);
-  v[V_SP * kNNode + i] = s_restr(M, T, tc, kk, true);
-  v[V_IP * kNNode + i] = init::lambda_ioni(M, T, tc, true);
-  v[V_BP * kNNode + i] = init::lambda_brem(M, T, kk);
-  v[V_AP * kNNode + i] = init::lambda_annih(M, T);
-  if (i < kNNode - 1) {
-    s.bins[((size_t)m * 3 + B_RE) * kNNode + i] = bin_integral(i, [&](double x) { return s_restr(M, x, tc, kk, false); });
-    s.bins[((size_t)m * 3 + B_RP) * kNNode + i] = bin_integral(i, [&](double x) { return s_restr(M, x, tc, kk, true); });
-  }
-}
-
-__global__ void k_ranges(const MatDev* mats, int n_mat, BuildScratch s) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 2 * n_mat) return;
-  const int m = idx >> 1, pos = idx & 1;
-  if (mats[m].vacuum) return;
-  double* v = s.vals + (size_t)m * V_NROW * kNNode;
-  init::prefix_range(v + (pos ? V_SP : V_SE) * kNNode, s.bins + ((size_t)m * 3 + (pos ? B_RP : B_RE)) * kNNode,
-               v + (pos ? V_RP : V_RE) * kNNode);
-}
+// material records in device memory
+struct RecordsAt {
+  const double* p;
+  __device__ const double* record(int m) const { return p + kMatRec * m; }
+};
 
 struct PackOut {
   double2 *g64, *e64, *p64;
@@ -175,11 +101,9 @@ cudaError_t launch_build_tables(const Params& P, const double* mat_in, int n_mat
                                 uint16_t* const range_index[4], double* Tc, double* kc, cudaStream_t st) {
   const int nn = n_mat * kNNode;
   const int B = 128;
-  k_materials<<<1, 32, 0, st>>>(mat_in, n_mat, mat);
-  k_gamma_full<<<(nn + B - 1) / B, B, 0, st>>>(mat, n_mat, s);
-  k_cuts<<<1, 32, 0, st>>>(mat, n_mat, range_cut, s, Tc, kc);
-  k_charged<<<(nn + B - 1) / B, B, 0, st>>>(mat, n_mat, s, Tc, kc);
-  k_ranges<<<1, 32, 0, st>>>(mat, n_mat, s);
+  const TableRows r{s.vals, (size_t)V_NROW * kNNode, s.bins, (size_t)B_NROW * kNNode, Tc, kc, 1, nullptr};
+  const cudaError_t e = launch_table_rows(RecordsAt{mat_in}, n_mat, range_cut, mat, r, st);
+  if (e != cudaSuccess) return e;
   PackOut o{g64, e64, p64, g32, e32, p32, re64, rp64, re32, rp32};
   k_pack<<<(nn + B - 1) / B, B, 0, st>>>(mat, n_mat, s, o, P.process_mask);
   // (last: the index takes the place of the bin integrals)

@@ -174,8 +174,20 @@ struct TrackIn {
 
 // ---- kernel launchers (kernels.cu) ----
 struct BuildScratch {
-  double* vals;     // [mat][16][kNNode] raw table values
-  double* bins;     // [mat][4][kNNode] per-bin range integrals
+  double* vals;     // [mat][14][kNNode] raw table values
+  double* bins;     // [mat][3][kNNode] per-bin range integrals
+};
+// Raw rows of a table build: 14 value rows of material m at v + m * v_stride (V_* in tables.cuh)
+// and three rows of bin integrals at b + m * b_stride; thresholds at Tc, kc + m * cut_stride.
+// out, if not null: the 12 tables of material m at out + m * 12 * kNNode (gamma, e-, e+).
+struct TableRows {
+  double* v;
+  size_t v_stride;
+  double* b;
+  size_t b_stride;
+  double *Tc, *kc;
+  int cut_stride;
+  double* out;
 };
 cudaError_t launch_build_tables(const Params& P, const double* mat_in, int n_mat, double range_cut,
                                 MatDev* mat, BuildScratch s, double2* g64, double2* e64, double2* p64,

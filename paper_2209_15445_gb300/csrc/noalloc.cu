@@ -1,7 +1,6 @@
 // adept_build_tables_noalloc: the physics-table build for callers that cannot allocate
-// device memory. Same closed forms and quadrature as adept_build_tables, fused into one
-// kernel (one block per material) whose working rows live in a file-scope __device__
-// array instead of a caller-provided arena.
+// device memory. The kernels of adept_build_tables' rows (tables.cuh), with their working rows
+// in a file-scope __device__ array instead of a caller-provided arena.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -9,88 +8,31 @@
 #include "../../include/adept.h"
 #include "device.cuh"
 #include "layout.h"
-#include "physics_init.cuh"
+#include "tables.cuh"
 
 namespace adept {
 namespace {
 
-constexpr int kRows = 17;  // 14 value rows + 3 rows of per-bin range integrals
+constexpr int kRows = V_NROW + B_NROW;
 constexpr int kNoAllocMat = ADEPT_NOALLOC_MAX_MATERIALS;
 
-// Working rows of every call, on every device that loads the library (held until exit):
-// kNoAllocMat x 17 x 289 doubles = 157 KB. Calls share it; each call writes every word it
-// reads before reading it, so nothing needs clearing, but calls that overlap on the GPU
-// race on it.
-static __device__ __align__(256) double g_noalloc_scratch[kNoAllocMat * kRows * kNNode];
+// Working rows and material constants of every call, on every device that loads the library
+// (held until exit): kNoAllocMat x 17 x 289 doubles = 157 KB. Calls share it; each call writes
+// every word it reads before reading it, so nothing needs clearing, but calls that overlap on
+// the GPU race on it.
+struct Scratch {
+  double rows[kNoAllocMat * kRows * kNNode];
+  MatDev mats[kNoAllocMat];
+};
+static __device__ __align__(256) Scratch g_noalloc_scratch;
 
 struct MatIn {
   double v[kNoAllocMat][kMatRec];  // material records (elements only), passed by value
+  __device__ const double* record(int m) const { return v[m]; }
 };
 
-enum { R_MUC, R_MUP, R_MUPH, R_SFULL, R_SE, R_IE, R_BE, R_SP, R_IP, R_BP, R_AP, R_RFULL, R_RE, R_RP, R_BFULL, R_BE_, R_BP_ };
-
-// one block per material; output tables [m][12][289] (gamma 3, e- 4, e+ 5) and cuts [m][2]
-__global__ void k_tables_noalloc(MatIn in, double range_cut, double* scratch, double* out, double* cuts) {
-  const int m = blockIdx.x;
-  __shared__ MatDev M;
-  __shared__ double tc, kc;
-  if (threadIdx.x == 0) init::setup_material(in.v[m], &M);
-  __syncthreads();
-  double* w = scratch + (size_t)m * kRows * kNNode;
-  double* o = out + (size_t)m * 12 * kNNode;
-  const int i = threadIdx.x;
-  if (M.vacuum) {
-    for (int k = i; k < 12 * kNNode; k += blockDim.x) o[k] = 0.0;
-    if (i == 0) { cuts[2 * m] = 0.0; cuts[2 * m + 1] = 0.0; }
-    return;
-  }
-  auto full = [&](double T) { return init::dedx_col(M, T, T, false) + init::dedx_rad(M, T, T); };
-  if (i < kNNode) {
-    const double E = init::node_E(i);
-    w[R_MUC * kNNode + i] = init::mu_compton(M, E);
-    w[R_MUP * kNNode + i] = init::mu_pair(M, E);
-    w[R_MUPH * kNNode + i] = init::mu_photo(M, E);
-    w[R_SFULL * kNNode + i] = full(E);
-    if (i < kNNode - 1) w[R_BFULL * kNNode + i] = init::bin_integral(i, full);
-  }
-  __syncthreads();
-  if (i == 0) {
-    init::prefix_range(w + R_SFULL * kNNode, w + R_BFULL * kNNode, w + R_RFULL * kNNode);
-    auto mu = [&](int k) { return w[R_MUC * kNNode + k] + w[R_MUP * kNNode + k] + w[R_MUPH * kNNode + k]; };
-    tc = init::clamp_cut(init::range_threshold(w + R_RFULL * kNNode, range_cut));
-    kc = init::clamp_cut(init::gamma_threshold(mu, range_cut));
-    cuts[2 * m] = tc;
-    cuts[2 * m + 1] = kc;
-  }
-  __syncthreads();
-  const double Tc = tc, Kc = kc;
-  auto se = [&](double T) { return init::dedx_col(M, T, Tc, false) + init::dedx_rad(M, T, Kc); };
-  auto sp = [&](double T) { return init::dedx_col(M, T, Tc, true) + init::dedx_rad(M, T, Kc); };
-  if (i < kNNode) {
-    const double T = init::node_E(i);
-    w[R_SE * kNNode + i] = se(T);
-    w[R_IE * kNNode + i] = init::lambda_ioni(M, T, Tc, false);
-    w[R_BE * kNNode + i] = init::lambda_brem(M, T, Kc);
-    w[R_SP * kNNode + i] = sp(T);
-    w[R_IP * kNNode + i] = init::lambda_ioni(M, T, Tc, true);
-    w[R_BP * kNNode + i] = init::lambda_brem(M, T, Kc);
-    w[R_AP * kNNode + i] = init::lambda_annih(M, T);
-    if (i < kNNode - 1) {
-      w[R_BE_ * kNNode + i] = init::bin_integral(i, se);
-      w[R_BP_ * kNNode + i] = init::bin_integral(i, sp);
-    }
-  }
-  __syncthreads();
-  if (i == 0) init::prefix_range(w + R_SE * kNNode, w + R_BE_ * kNNode, w + R_RE * kNNode);
-  if (i == 1) init::prefix_range(w + R_SP * kNNode, w + R_BP_ * kNNode, w + R_RP * kNNode);
-  __syncthreads();
-  const int rows[12] = {R_MUC, R_MUP, R_MUPH, R_SE, R_RE, R_IE, R_BE, R_SP, R_RP, R_IP, R_BP, R_AP};
-  if (i < kNNode)
-    for (int r = 0; r < 12; ++r) o[r * kNNode + i] = w[rows[r] * kNNode + i];
-}
-
 std::mutex g_mu;
-double* g_ptr[256] = {};
+Scratch* g_ptr[256] = {};
 
 }  // namespace
 }  // namespace adept
@@ -111,7 +53,7 @@ extern "C" int adept_build_tables_noalloc(const adept_material* materials, int32
   }
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return ADEPT_ECUDA;
-  double* scratch;
+  Scratch* scratch;
   {
     // the array's device address, once per device with that device current; host code
     // cannot use the symbol itself (it names a host-side stand-in)
@@ -119,11 +61,12 @@ extern "C" int adept_build_tables_noalloc(const adept_material* materials, int32
     if (!g_ptr[dev]) {
       void* p = nullptr;
       if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return ADEPT_ECUDA;
-      g_ptr[dev] = static_cast<double*>(p);
+      g_ptr[dev] = static_cast<Scratch*>(p);
     }
     scratch = g_ptr[dev];
   }
-  k_tables_noalloc<<<n_materials, 320, 0, static_cast<cudaStream_t>(stream)>>>(in, range_cut_mm, scratch, dev_tables,
-                                                                               dev_cuts);
-  return cudaGetLastError() == cudaSuccess ? ADEPT_OK : ADEPT_ECUDA;
+  const TableRows r{scratch->rows, (size_t)kRows * kNNode, scratch->rows + V_NROW * kNNode, (size_t)kRows * kNNode,
+                    dev_cuts, dev_cuts + 1, 2, dev_tables};
+  return launch_table_rows(in, n_materials, range_cut_mm, scratch->mats, r, static_cast<cudaStream_t>(stream)) == cudaSuccess
+             ? ADEPT_OK : ADEPT_ECUDA;
 }

@@ -13,10 +13,20 @@ namespace init {
 // so below k = 0.2 b is taken from its Taylor series in x = 2k instead: term by term from
 // the expansions of ln(1+x), 1/(1+x) and 1/(1+x)^2, b = sum_n (-x)^n d_n with
 // d_n = 4(n+1)/(n+3) + 1/(n+1) - 2n/(n+2) + n/2 - 1 (d_0 = 4/3, Thomson), 60 terms.
-__device__ inline double kn_series_term(int n) {
+// The coefficients are constants: computed on the device, their 180 divisions were the longest
+// chain of the table build (one thread a node).
+constexpr double kn_series_term(int n) {
   const double dn = (double)n;
   return 4.0 * (dn + 1.0) / (dn + 3.0) + 1.0 / (dn + 1.0) - 2.0 * dn / (dn + 2.0) + 0.5 * dn - 1.0;
 }
+constexpr int kKnTerms = 60;
+struct KnSeries {
+  double d[kKnTerms];
+  constexpr KnSeries() : d() {
+    for (int n = 0; n < kKnTerms; ++n) d[n] = kn_series_term(n);
+  }
+};
+static __constant__ KnSeries kKnSeries;
 __device__ inline double sigma_kn(double k) {
   double b;
   if (k >= 0.2) {
@@ -25,8 +35,9 @@ __device__ inline double sigma_kn(double k) {
     b = (1.0 + k) / (k * k) * (2.0 * (1.0 + k) / a - l / k) + l / (2.0 * k) - (1.0 + 3.0 * k) / (a * a);
   } else {
     const double mx = -2.0 * k;
-    b = kn_series_term(59);
-    for (int n = 58; n >= 0; --n) b = fma(b, mx, kn_series_term(n));
+    b = kKnSeries.d[kKnTerms - 1];
+#pragma unroll
+    for (int n = kKnTerms - 2; n >= 0; --n) b = fma(b, mx, kKnSeries.d[n]);
   }
   return 2.0 * kPi * kRe * kRe * b;
 }
@@ -194,30 +205,35 @@ __device__ inline double lambda_annih(const MatDev& m, double T) {
 }
 
 // ---------------------------------------------------------------- range and thresholds
-// Shared by the arena build (kernels.cu) and the allocation-free build (noalloc.cu), so
-// that both builds follow one set of rules.
-
 // energy of grid node i
 __device__ inline double node_E(int i) { return exp(kLnEmin + (double)i * kDlog); }
 
-// Simpson rule with 8 panels of T/S(T) over bin i in ln T: the range gained across bin i
+// Simpson rule with 8 panels of T/S(T) over bin i in ln T: the range gained across bin i. One
+// warp takes three bins, a lane for each of a bin's nine points, and adds the points up in
+// order. Every lane of the warp calls this; lane 9k of bin k (k < 3) gets its integral.
+constexpr int kBinsPerWarp = 3, kSimpson = 9;
 template <class F>
-__device__ inline double bin_integral(int i, F S) {
+__device__ inline double warp_bin_integral(int first_bin, F S) {
+  const int lane = threadIdx.x & 31, k = lane / kSimpson, j = lane % kSimpson;
+  const int i = first_bin + k;
   const double h = kDlog / 8.0;
-  double acc = 0.0;
-  for (int j = 0; j <= 8; ++j) {
+  double term = 0.0;
+  if (k < kBinsPerWarp && i < kNNode - 1) {
     const double T = exp(kLnEmin + (double)i * kDlog + (double)j * h);
     const double w = (j == 0 || j == 8) ? 1.0 : ((j & 1) ? 4.0 : 2.0);
-    acc += w * (T / S(T));
+    term = w * (T / S(T));
   }
+  double acc = 0.0;
+  for (int n = 0; n < kSimpson; ++n) acc += __shfl_sync(0xFFFFFFFFu, term, (k * kSimpson + n) & 31);
   return acc * h / 3.0;
 }
 
-// range of a stopping-power row: R(E0) = E0/(2 S(E0)) (S taken as 1/T below the grid),
-// then the running sum of the bin integrals
-__device__ inline void prefix_range(const double* S, const double* bins, double* R) {
-  double r = node_E(0) / (2.0 * S[0]);
+// range of a stopping-power row: R(E0) = E0/(2 S(E0)) (S taken as 1/T below the grid, s0 = S(E0)),
+// then the running sum of the bin integrals, in order (bins and R in shared memory)
+__device__ inline void prefix_range(double s0, const double* bins, double* R) {
+  double r = node_E(0) / (2.0 * s0);
   R[0] = r;
+#pragma unroll 8
   for (int i = 0; i < kNNode - 1; ++i) {
     r += bins[i];
     R[i + 1] = r;
@@ -228,29 +244,23 @@ __device__ inline void prefix_range(const double* S, const double* bins, double*
 __device__ inline double clamp_cut(double x) { return x < 0.99e-3 ? 0.99e-3 : (x > 1e4 ? 1e4 : x); }
 
 // e+- threshold: the energy whose unrestricted range R (node values, rising) equals the
-// range cut, by exact inversion of the range interpolated linearly in ln E
-__device__ inline double range_threshold(const double* R, double range_cut) {
+// range cut, by exact inversion of the range interpolated linearly in ln E; i is the first
+// interval whose end reaches the cut (kNNode - 1: none)
+__device__ inline double range_threshold(const double* R, double range_cut, int i) {
   if (range_cut <= R[0]) return node_E(0);
-  for (int i = 0; i < kNNode - 1; ++i)
-    if (R[i + 1] >= range_cut) {
-      const double t = (range_cut - R[i]) / (R[i + 1] - R[i]);
-      return exp(kLnEmin + ((double)i + t) * kDlog);
-    }
-  return 1e6;
+  if (i >= kNNode - 1) return 1e6;
+  const double t = (range_cut - R[i]) / (R[i + 1] - R[i]);
+  return exp(kLnEmin + ((double)i + t) * kDlog);
 }
 
-// gamma threshold: five mean free paths equal the range cut, on the falling low-energy
-// branch of the total attenuation mu(i) (node values)
-template <class F>
-__device__ inline double gamma_threshold(F mu, double range_cut) {
-  const double target = 5.0 / range_cut;
-  if (mu(0) <= target) return node_E(0);
-  for (int i = 0; i < kNNode - 1; ++i)
-    if (mu(i + 1) <= target) {
-      const double a = mu(i), b = mu(i + 1);
-      return exp(kLnEmin + ((double)i + (a - target) / (a - b)) * kDlog);
-    }
-  return 1e6;
+// gamma threshold: five mean free paths equal the range cut (target = 5 / cut), on the falling
+// low-energy branch of the total attenuation mu (node values); i is the first interval whose
+// end is at or below the target
+__device__ inline double gamma_threshold(const double* mu, double target, int i) {
+  if (mu[0] <= target) return node_E(0);
+  if (i >= kNNode - 1) return 1e6;
+  const double a = mu[i], b = mu[i + 1];
+  return exp(kLnEmin + ((double)i + (a - target) / (a - b)) * kDlog);
 }
 
 }  // namespace init
