@@ -410,6 +410,7 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   P.geo.safe_z = (float)(geometry->half_length_mm * 0.9999 - 2.0);
   P.geo.bnd = bnd; P.geo.vol_mat = vm; P.geo.vol_bin = vb;
   P.mat = c->mat_dev;
+  P.n_mat = c->n_mat;
   P.tab = TableView{c->g64, c->e64, c->p64, c->g32, c->e32, c->p32, c->re64, c->rp64, c->re32, c->rp32,
                     c->xr[0], c->xr[1], c->xr[2], c->xr[3], c->Tc, c->kc};
   E.max_slots = ms;
@@ -481,7 +482,10 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
       int bps = transport_max_blocks_per_sm(o.precision, sp, c->minb[sp], o.block_size, transport_variant(P));
       c->grid[sp] = sms * (bps < 1 ? 1 : bps);
     }
-    if (c->tail_tracks) c->tail_blocks = tail_blocks(P, o.precision, o.fused != 0);
+    if (c->tail_tracks) {
+      P.tail_shared = tail_shared_bytes(P, o.precision, o.fused != 0);
+      c->tail_blocks = tail_blocks(P, o.precision, o.fused != 0);
+    }
     if (o.fused) {
       int mb = o.blocks_per_sm > 0 ? o.blocks_per_sm : (o.precision ? 2 : 1);
       c->fminb = std::min(4, mb);

@@ -132,6 +132,7 @@ struct EventView {
 struct Params {
   GeoView geo;
   const MatDev* mat;
+  int n_mat;
   TableView tab;
   char* queues;         // the six track queues (see Tile), queue_bytes apart
   size_t queue_bytes;
@@ -153,6 +154,7 @@ struct Params {
   double delta_chord;   // chord sagitta limit, mm
   double delta_int;     // intersection accuracy, mm
   uint32_t tail_exit;   // a tail chunk ends once this many tracks are live
+  uint32_t tail_shared; // bytes of a tail block's copy of the tables and the geometry (0: none)
   // the host's pinned, device-mapped status of the two chunk buffers: the copy of Ctrl and the
   // done list ([evt.max_slots]: slots found finished) that a chunk's finish pass writes, and the
   // outgoing-ring read position its first kernel reads (so no copy sits between two chunks)
@@ -204,7 +206,9 @@ constexpr uint32_t kGkDevice = 0xFFFFFFFFu;
 // 4.62, 5.1. FP64, whose generations want more SMs: 10 showers 6.8 (512 to 2048), 8.4 (8192).
 constexpr uint32_t kTailTracks = 12288, kTailTracksFp64 = 2048;
 cudaError_t launch_tail(const Params& P, int precision, bool fused, int blocks, uint32_t max_gens, cudaStream_t st);
-// blocks of its cluster (one a species in turn): 16, or 8 where no cluster of 16 can be resident
+// the bytes for Params::tail_shared, and then the blocks of its cluster (one a species in turn):
+// 16, or 8 where no cluster of 16 can be resident
+uint32_t tail_shared_bytes(const Params& P, int precision, bool fused);
 int tail_blocks(const Params& P, int precision, bool fused);
 // its kernels with chords, and with the step-length histogram
 const void* tail_variant_fn(int precision, int variant);

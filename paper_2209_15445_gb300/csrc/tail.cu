@@ -3,6 +3,8 @@
 // with the fused one, and the launch of every variant's.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "layout.h"
 #include "tail.cuh"
 
@@ -15,8 +17,9 @@ static const void* tail_fn(int variant, bool fused) {
   return (variant & 8) ? (const void*)k_tail<R, 0, 8> : (const void*)k_tail<R, 0, 0>;
 }
 
-static void tail_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int blocks, cudaStream_t st) {
+static void tail_config(const Params& P, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int blocks, cudaStream_t st) {
   cfg = {};
+  cfg.dynamicSmemBytes = P.tail_shared;
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(256);
   cfg.stream = st;
@@ -31,11 +34,26 @@ static const void* tail_fn(const Params& P, int precision, bool fused) {
   return precision ? tail_fn<float>(transport_variant(P), fused) : tail_fn<double>(transport_variant(P), fused);
 }
 
+uint32_t tail_shared_bytes(const Params& P, int precision, bool fused) {
+  uint32_t n = 0;
+  for (int s = 0; s < 3; ++s) n = std::max(n, precision ? tail_units<float>(P, s) : tail_units<double>(P, s));
+  const void* fn = tail_fn(P, precision, fused);
+  cudaFuncAttributes fa;
+  int dev = 0, most = 0;
+  if (cudaFuncGetAttributes(&fa, fn) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+      16u * n + fa.sharedSizeBytes <= (size_t)most &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(16u * n)) == cudaSuccess)
+    return 16u * n;
+  (void)cudaGetLastError();
+  return 0;  // too many materials or volumes: read where they are
+}
+
 int tail_blocks(const Params& P, int precision, bool fused) {
   const void* fn = tail_fn(P, precision, fused);
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at;
-  tail_config(cfg, at, 16, nullptr);
+  tail_config(P, cfg, at, 16, nullptr);
   int n = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
       cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0)
@@ -48,7 +66,7 @@ cudaError_t launch_tail(const Params& P, int precision, bool fused, int blocks, 
   void* args[] = {const_cast<Params*>(&P), &max_gens};
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at;
-  tail_config(cfg, at, blocks, st);
+  tail_config(P, cfg, at, blocks, st);
   return cudaLaunchKernelExC(&cfg, tail_fn(P, precision, fused), args);
 }
 

@@ -151,8 +151,8 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
   const double rest = S == 2 ? 2.0 * kMe : 0.0;
   const int vol = (int)(t.nav & 0xFFFFu);
   uint32_t vac = t.nav >> 16;
-  const int m = __ldg(P.geo.vol_mat + vol);
-  dep_bin = __ldg(P.geo.vol_bin + vol);
+  const int m = ro(P.geo.vol_mat + vol);
+  dep_bin = ro(P.geo.vol_bin + vol);
   sec.n = 0;
   dep = 0.0;
   const uint32_t step = t.step;
@@ -248,7 +248,7 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
       t.z += to_d<R>(s * t.u[2]);
     }
   }
-  if (boundary && P.geo.kind == 0 && next >= 0) t.z = __ldg(P.geo.bnd + (t.u[2] > (R)0 ? vol + 1 : vol));
+  if (boundary && P.geo.kind == 0 && next >= 0) t.z = ro(P.geo.bnd + (t.u[2] > (R)0 ? vol + 1 : vol));
   t.step = step + 1;
   if constexpr ((V & 4) != 0) {
     if (P.steplen && s > (R)0 && s < M<R>::big()) {
@@ -270,7 +270,7 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
     if constexpr (PH) {
       if (fluct && s < Rr && Ep >= P.tcut) {
         const R xi = (R)(kTwoPiRe2Me * __ldg(&P.mat[m].n_el));
-        const R sig = M<R>::sqrt(fluct_sigma2<R>(Er, xi, (R)__ldg(P.tab.Tc + m), s, S == 2));
+        const R sig = M<R>::sqrt(fluct_sigma2<R>(Er, xi, (R)ro(P.tab.Tc + m), s, S == 2));
         Ep = t.E - fluct_loss<R>(rs, t.E - Ep, sig);
         Epr = to_r<R>(Ep);
       }
@@ -328,8 +328,8 @@ __device__ __forceinline__ bool step_interact(const Params& P, Trk<R>& t, uint32
     annihilate_at_rest<R>(rs, sec);
     return false;
   }
-  const int m = __ldg(P.geo.vol_mat + (int)(t.nav & 0xFFFFu));
-  const double Tc = __ldg(P.tab.Tc + m), kc = __ldg(P.tab.kc + m);
+  const int m = ro(P.geo.vol_mat + (int)(t.nav & 0xFFFFu));
+  const double Tc = ro(P.tab.Tc + m), kc = ro(P.tab.kc + m);
   const R tcut = (R)P.tcut;
   sec.happened = false;
   sec.n = 0;
@@ -504,7 +504,7 @@ __device__ __forceinline__ void run_tiles(const Params& P, int p, int cw, uint32
       pstep = ring.pstep[j];
       t.step = pstep + 1;
       outcome = step_interact<R, S>(P, t, pstep, (int)(nv >> 16), sec, dep) ? kAlive : kDead;
-      bin = __ldg(P.geo.vol_bin + (int)(t.nav & 0xFFFFu));
+      bin = ro(P.geo.vol_bin + (int)(t.nav & 0xFFFFu));
     }
     // S10: score the step's deposit in (event, layer, material)
     score(P, t.ev, bin, dep);

@@ -13,12 +13,21 @@ from gpu_common import make, need_gpu
 pytestmark = pytest.mark.gpu
 
 SLAB, BARREL = W.slab_calorimeter, W.barrel_calorimeter
+
+
+def EIGHT():
+    """eight materials: in FP64 their tables do not fit a block's shared memory beside its rings"""
+    mats = [W.PB, W.LAR, W.SI, W.FE, W.PBWO4, W.PB, W.FE, W.SI]
+    return W.Geometry(kind=0, n_layers=12, materials=mats, sub_materials=list(range(8)),
+                      sub_thickness=[2.0, 3.0, 0.3, 2.0, 2.0, 1.0, 1.0, 4.0], half_xy=200.0)
+
+
 VARIANTS = [("plain", SLAB, {}), ("field", SLAB, dict(field_T=1.0)), ("barrel", BARREL, dict(field_T=3.8)),
             ("msc", SLAB, dict(physics=1)), ("msc_fluct_field", BARREL, dict(physics=3, field_T=3.8)),
             ("chords", BARREL, dict(field_T=3.8, field_max_iterations=100, max_steps=300)),
             ("chords_msc", BARREL, dict(field_T=3.8, field_max_iterations=50, physics=1, max_steps=300)),
             ("histogram", SLAB, dict(flags=8)), ("histogram_field", BARREL, dict(flags=8, field_T=3.8)),
-            ("fused", SLAB, dict(fused=1))]
+            ("fused", SLAB, dict(fused=1)), ("eight_materials", EIGHT, {})]
 
 
 @pytest.mark.parametrize("precision", [0, 1])
