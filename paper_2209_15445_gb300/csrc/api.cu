@@ -417,6 +417,7 @@ extern "C" int adept_init(adept_ctx** out, const adept_geometry* geometry, const
   P.max_log = o.max_generation_log;
   P.field_T = cuts->field_T;
   P.tcut = cuts->tracking_cut_MeV;
+  for (uint32_t r = 0; r < 10; ++r) P.seed_keys[r] = o.seed + r * 0x9E3779B9u;
   P.seed = o.seed; P.process_mask = o.process_mask; P.max_steps = o.max_steps; P.max_vac = o.max_vacuum_steps;
   P.steplen = (o.flags & ADEPT_FLAG_STEP_HISTOGRAM) ? steplen : nullptr;
   P.physics = o.physics;

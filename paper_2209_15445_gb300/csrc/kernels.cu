@@ -469,7 +469,7 @@ template <class R>
 __global__ void k_probe_sample(Params P, int which, int m, double E, uint32_t event, int n, double* out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  Stream<R> st(P.seed, event, (unsigned long long)(i + 1), 0u);
+  Stream<R> st(P, event, (unsigned long long)(i + 1), 0u);
   const R u[3] = {(R)0, (R)0, (R)1};
   Ixn<R> r;
   r.happened = false; r.parent_alive = false; r.n = 0; r.parent_E = 0.0;
@@ -510,7 +510,7 @@ __global__ void k_probe_continuous(Params P, int which, int species, int m, doub
                                    double* out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  Stream<R> st(P.seed, event, (unsigned long long)(i + 1), 0u);
+  Stream<R> st(P, event, (unsigned long long)(i + 1), 0u);
   const MatDev& md = P.mat[m];
   if (which == 0) {
     R u[3] = {(R)0, (R)0, (R)1};

@@ -145,6 +145,7 @@ struct Params {
   double field_T;
   double tcut;
   uint32_t seed, process_mask, max_steps, max_vac;
+  uint32_t seed_keys[10];  // seed + r * 0x9E3779B9: the seed's share of Philox's round keys
   unsigned long long* steplen;  // [3][64] step-length histogram (log2 bins), or null
   uint32_t physics;     // ADEPT_PHYS_* bits: multiple scattering, loss fluctuations
   double msc_f;         // multiple-scattering step limit: s <= max(msc_f R, 0.01 mm)

@@ -166,7 +166,7 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
   }
   const R tcut = (R)P.tcut;
   const R Er = to_r<R>(t.E);
-  Stream<R> rs(P.seed, __ldg(P.evt.key + t.ev), t.id, step);
+  Stream<R> rs(P, __ldg(P.evt.key + t.ev), t.id, step);
   if (Er < tcut) {
     dep = t.E;
     if (S == 2) { proc = 3; return kInteract; }  // annihilates at rest in phase B
@@ -313,7 +313,7 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
 template <class R, int S>
 __device__ __forceinline__ bool step_interact(const Params& P, Trk<R>& t, uint32_t pstep, int proc, Ixn<R>& sec,
                                               double& dep) {
-  Stream<R> rs(P.seed, __ldg(P.evt.key + t.ev), t.id, pstep);
+  Stream<R> rs(P, __ldg(P.evt.key + t.ev), t.id, pstep);
   if (proc == 4) {  // the track left the world: its energy and its outgoing record
     sec.happened = false;
     sec.n = 0;
@@ -425,7 +425,7 @@ __device__ __forceinline__ void emit(const Params& P, int p, int cw, const Trk<R
     const uint32_t mine = __popc((k == 0 ? pick(b1, sk) : pick(b2, sk)) & lt);
     const uint32_t d = pick(wbase, sk) + before + mine;
     if (d < P.cap) {
-      const unsigned long long cid = child_id(P.seed, __ldg(P.evt.key + t.ev), t.id, pstep, (uint32_t)k);
+      const unsigned long long cid = child_id(P, __ldg(P.evt.key + t.ev), t.id, pstep, (uint32_t)k);
       store_track<R>(track_queue(P, p ^ 1, sk), d, t.x, t.y, t.z, sec.d[k][0], sec.d[k][1], sec.d[k][2], sec.E[k], cid, t.ev, 0u,
                      vnav);
     } else {
