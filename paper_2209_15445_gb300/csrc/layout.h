@@ -33,6 +33,7 @@ constexpr int kMatRec = 5 + 3 * kMaxElem;      // material record: Z, A, rho, I,
 
 struct MatDev {
   double Z, A, rho, I;   // I in eV (a compound: its mean Z and A)
+  double mass_per_mm;    // mass thickness of 1 mm, g/cm^2
   int n_elem;            // elements: Z and atoms per mm^3
   double eZ[kMaxElem], en_at[kMaxElem];
   double ZoA;            // <Z/A> by mass

@@ -56,6 +56,7 @@ __device__ inline double inv_x0_per_atom(double Z) {
 // the formula's mass fractions.
 __device__ inline void setup_material(const double* in, MatDev* m) {
   m->Z = in[0]; m->A = in[1]; m->rho = in[2]; m->I = in[3];
+  m->mass_per_mm = 0.1 * m->rho;
   const int ne = (int)in[4];
   m->vacuum = !(m->Z > 0.0) && ne == 0;
   m->n_elem = 0;
