@@ -172,6 +172,7 @@ struct adept_ctx {
   std::unordered_map<uint32_t, std::unique_ptr<Request>> reqs;
   std::vector<Request*> slot_req;  // slot -> its request while that is in flight (else null)
   SlotAlloc slots;
+  uint32_t slot_end = 0;  // past the highest slot admitted since none was in flight
   double energy_in_flight = 0.0;
   size_t in_flight = 0;
   adept_stats stats{};
@@ -664,6 +665,7 @@ static int admit(adept_ctx* c) {
       r->state = 1;
       r->remaining = (uint32_t)r->keys.size();
       for (uint32_t k = 0; k < r->remaining; ++k) c->slot_req[base + k] = r;
+      c->slot_end = std::max(c->in_flight ? c->slot_end : 0u, base + r->remaining);
       c->energy_in_flight += r->energy;
       c->in_flight++;
       c->admit_est += (uint64_t)(r->energy * c->opt.tracks_per_MeV) + r->n;
@@ -789,10 +791,9 @@ static int launch_chunk(adept_ctx* c, int b) {
   c->tail[b] = G > 0 && live < (uint64_t)c->tail_tracks;
   c->admit_mark[b] = c->admit_est;
   if (c->tail[b]) {
-    CK(launch_open_chunk(c->P, b, c->stream));
-    CK(launch_tail(c->P, c->opt.precision, c->opt.fused != 0, c->tail_blocks, (uint32_t)gens, c->stream));
-    CK(launch_finish(c->P, b, kGkDevice, c->stream));
-    c->stats.launches += 5;  // chunk open, tail, end of chunk, mark, finish
+    CK(launch_tail(c->P, c->opt.precision, c->opt.fused != 0, c->tail_blocks, (uint32_t)gens, b, c->stream));
+    CK(launch_done(c->P, b, c->slot_end, c->stream));
+    c->stats.launches += 2;
   } else if (G > 0) {
     if (!c->graph[b]) {
       int rc = capture_graph(c, G, b);

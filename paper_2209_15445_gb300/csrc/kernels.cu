@@ -228,6 +228,7 @@ __global__ void k_init_primaries(Params P, const TrackIn* recs, const uint32_t* 
     atomicAdd(P.evt.killed + slot, r.E + rest);
     return;
   }
+  P.evt.alive[slot] = gen;  // as a chunk's marks would say (a tail chunk may mark none)
   store_track<R>(track_queue(P, p, sp), d, r.pos[0], r.pos[1], r.pos[2], (R)r.dir[0], (R)r.dir[1], (R)r.dir[2], r.E,
                  (unsigned long long)id, slot, 0u, (uint32_t)vol);
 }
@@ -241,38 +242,15 @@ cudaError_t launch_init_primaries(const Params& P, const TrackIn* recs, const ui
 }
 
 // ======================================================================== completion
-// End of a chunk of `gens` generations: log the sizes its last generation left, and advance
-// gen and the generation count. One thread.
 __global__ void k_end_chunk(Params P, uint32_t gens) {
-  if (threadIdx.x != 0) return;
-  volatile Ctrl* c = P.ctrl;
-  if (gens == kGkDevice) gens = c->tail_k;
-  if (gens == 0) return;  // a tail chunk that found the queues empty ran nothing
-  const uint32_t gen = c->gen + gens;
-  const uint32_t ln = c->log_n;
-  if (ln < P.max_log) {
-    for (int k = 0; k < 3; ++k) P.gen_log[3 * ln + k] = min(c->count[gen % 3][k].n, P.cap);
-    c->log_n = ln + 1;
-  }
-  c->generations = c->generations + gens;
-  c->gen = gen;
+  if (threadIdx.x == 0) close_chunk(P, __ldcg(&P.ctrl->gen), gens);
 }
 
 // An event is finished when no live track of it is left in the current queues: mark
 // the slots that still have tracks with the current generation, then every active slot
 // not marked is done and goes to the done list.
 __global__ void k_mark(Params P) {
-  const uint32_t gen = __ldcg(&P.ctrl->gen);
-  const int p = gen & 1, cr = gen % 3;
-  const uint32_t n0 = min(__ldcg(&P.ctrl->count[cr][0].n), P.cap), n1 = min(__ldcg(&P.ctrl->count[cr][1].n), P.cap),
-                 n2 = min(__ldcg(&P.ctrl->count[cr][2].n), P.cap);
-  const uint32_t total = n0 + n1 + n2;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const int sp = i < n0 ? 0 : (i < n0 + n1 ? 1 : 2);
-    const uint32_t j = sp == 0 ? i : (sp == 1 ? i - n0 : i - n0 - n1);
-    const uint32_t ev = track_event(P, track_queue(P, p, sp), j);
-    if (P.evt.alive[ev] != gen) P.evt.alive[ev] = gen;
-  }
+  mark_events(P, __ldcg(&P.ctrl->gen), blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // The same marks with per-block deduplication: a block sets one bit per event slot seen among
@@ -293,12 +271,7 @@ __global__ void k_mark_bits(Params P) {
   const uint32_t total = n0 + n1 + n2;
   if (blockIdx.x * blockDim.x >= total) return;  // a block with no tracks has nothing to mark
   if (total <= kMarkDirectTracks) {  // few tracks contend little: mark directly, as k_mark does
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-      const int sp = i < n0 ? 0 : (i < n0 + n1 ? 1 : 2);
-      const uint32_t j = sp == 0 ? i : (sp == 1 ? i - n0 : i - n0 - n1);
-      const uint32_t ev = track_event(P, track_queue(P, p, sp), j);
-      if (P.evt.alive[ev] != gen) P.evt.alive[ev] = gen;
-    }
+    mark_events(P, gen, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
     return;
   }
   const uint32_t nw = (P.evt.max_slots + 31u) / 32u;
@@ -319,9 +292,10 @@ __global__ void k_mark_bits(Params P) {
 // buffer b; the last block to end then writes the whole Ctrl there. The host reads both once
 // the chunk has ended, and no copy runs between two chunks (two device-to-host copies and one
 // host-to-device copy a chunk boundary before, and a synchronous one for long lists).
-__global__ void k_finish(Params P, int b) {
+// slots: event slots in use (all, or up to the highest admitted).
+__global__ void k_finish(Params P, int b, uint32_t slots) {
   const uint32_t gen = __ldcg(&P.ctrl->gen);
-  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < P.evt.max_slots; s += gridDim.x * blockDim.x) {
+  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < slots; s += gridDim.x * blockDim.x) {
     if (P.evt.state[s] == 1u && P.evt.alive[s] != gen) {
       P.evt.state[s] = 2u;
       P.h_done[b][atomicAdd(&P.ctrl->done_count[b], 1u)] = s;
@@ -341,16 +315,18 @@ __global__ void k_finish(Params P, int b) {
   __threadfence_system();
 }
 
-// Start of a chunk: the outgoing-ring read position the host left in its pinned copy of
-// buffer b, and an empty done count for the chunk's finish pass. One thread.
 __global__ void k_open_chunk(Params P, int b) {
-  if (threadIdx.x != 0) return;
-  P.ctrl->leak_floor = *reinterpret_cast<const volatile unsigned long long*>(P.h_floor[b]);
-  P.ctrl->done_count[b] = 0;
+  if (threadIdx.x == 0) open_chunk(P, b);
 }
 
 cudaError_t launch_open_chunk(const Params& P, int b, cudaStream_t st) {
   k_open_chunk<<<1, 32, 0, st>>>(P, b);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_done(const Params& P, int b, uint32_t slots, cudaStream_t st) {
+  const uint32_t blocks = (slots + 255) / 256;
+  k_finish<<<blocks < 1 ? 1 : (blocks < 1216 ? blocks : 1216), 256, 0, st>>>(P, b, slots);
   return cudaGetLastError();
 }
 
@@ -360,8 +336,7 @@ cudaError_t launch_finish(const Params& P, int b, uint32_t gens, cudaStream_t st
     k_mark_bits<<<304, 512, sizeof(uint32_t) * ((P.evt.max_slots + 31) / 32), st>>>(P);
   else
     k_mark<<<1216, 256, 0, st>>>(P);
-  k_finish<<<(P.evt.max_slots + 255) / 256 < 1216 ? (P.evt.max_slots + 255) / 256 : 1216, 256, 0, st>>>(P, b);
-  return cudaGetLastError();
+  return launch_done(P, b, P.evt.max_slots, st);
 }
 
 // ======================================================================== probes

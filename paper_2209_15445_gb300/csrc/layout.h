@@ -98,7 +98,7 @@ struct Ctrl {
   uint32_t done_count[2];     // events found finished by the finish pass of a chunk (per buffer)
   uint32_t log_n;             // rows written to the generation log
   uint32_t error;             // first device-detected error code (0 = none)
-  uint32_t tail_k;            // generations the last tail chunk ran (see kGkDevice)
+  uint32_t tail_k;            // generations the last tail chunk ran
   uint32_t finish_ticket;     // blocks of the finish pass that have ended (the last one resets it)
   uint32_t pad[2];
   unsigned long long steps[3];
@@ -198,16 +198,15 @@ cudaError_t launch_build_tables(const Params& P, const double* mat_in, int n_mat
                                 float2* g32, float2* e32, float2* p32, double* re64, double* rp64,
                                 float* re32, float* rp32, uint16_t* const range_index[4], double* Tc, double* kc,
                                 cudaStream_t st);
-// A tail chunk: up to max_gens generations in one launch (tail.cuh), fewer if the queues run
-// empty or P.tail_exit tracks are live; the count is left in Ctrl::tail_k, which the end of the
-// chunk reads when its gens is kGkDevice.
-constexpr uint32_t kGkDevice = 0xFFFFFFFFu;
+// A tail chunk in status buffer b: up to max_gens generations in one launch (tail.cuh), fewer if
+// the queues run empty or P.tail_exit tracks are live, with the start and the end of a chunk but
+// for launch_done. Ctrl::tail_k gets the count.
 // It takes over below kTailTracks live tracks and ends at twice as many. Where the lines lie
 // (ms, by kTailTracks): 10 showers of 10 GeV 2.20 (4096), 2.13 (8192), 2.04 (16384), 2.38 with
 // fixed chunks; 100 showers 2.84, 2.84, 2.75, 3.15; a round of 16 serving requests 4.55, 4.56,
 // 4.62, 5.1. FP64, whose generations want more SMs: 10 showers 6.8 (512 to 2048), 8.4 (8192).
 constexpr uint32_t kTailTracks = 12288, kTailTracksFp64 = 2048;
-cudaError_t launch_tail(const Params& P, int precision, bool fused, int blocks, uint32_t max_gens, cudaStream_t st);
+cudaError_t launch_tail(const Params& P, int precision, bool fused, int blocks, uint32_t max_gens, int b, cudaStream_t st);
 // the bytes for Params::tail_shared, and then the blocks of its cluster (one a species in turn):
 // 16, or 8 where no cluster of 16 can be resident
 uint32_t tail_shared_bytes(const Params& P, int precision, bool fused);
@@ -226,10 +225,12 @@ cudaError_t launch_init_primaries(const Params& P, const TrackIn* recs, const ui
                                   uint32_t slot_base, int precision, cudaStream_t st);
 // start of a chunk in status buffer b: the host's outgoing-ring read position, done count 0
 cudaError_t launch_open_chunk(const Params& P, int b, cudaStream_t st);
-// end of a chunk of `gens` generations (kGkDevice: the count a tail chunk left in
-// Ctrl::tail_k): log the last one, advance gen, find finished events, and write the status
-// and the done list to the host's copy of buffer b
+// end of a chunk of `gens` generations: log the last one, advance gen, mark the events that have
+// tracks, and the pass of launch_done
 cudaError_t launch_finish(const Params& P, int buffer, uint32_t gens, cudaStream_t st);
+// find finished events among the first `slots`, and write the status and the done list to the
+// host's copy of buffer b
+cudaError_t launch_done(const Params& P, int b, uint32_t slots, cudaStream_t st);
 cudaError_t launch_probe_philox(const uint32_t* ctr, int n, uint32_t k0, uint32_t k1, uint32_t* out,
                                 cudaStream_t st);
 cudaError_t launch_probe_interp(const Params& P, int s, int t, int m, int prec, const double* E, int n,

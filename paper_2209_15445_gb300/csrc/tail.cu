@@ -62,8 +62,8 @@ int tail_blocks(const Params& P, int precision, bool fused) {
   return 8;
 }
 
-cudaError_t launch_tail(const Params& P, int precision, bool fused, int blocks, uint32_t max_gens, cudaStream_t st) {
-  void* args[] = {const_cast<Params*>(&P), &max_gens};
+cudaError_t launch_tail(const Params& P, int precision, bool fused, int blocks, uint32_t max_gens, int b, cudaStream_t st) {
+  void* args[] = {const_cast<Params*>(&P), &max_gens, &b};
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at;
   tail_config(P, cfg, at, blocks, st);

@@ -81,6 +81,7 @@ __device__ __forceinline__ uint32_t tail_species(Params P, uint32_t gen0, uint32
                                                  uint32_t count, WarpRing<R>& ring, uint32_t* nsteps, uint32_t* ncreated) {
   const uint32_t wpb = blockDim.x >> 5;
   if (P.tail_shared) stage_tables<R, S>(P);
+  cluster_sync();  // the chunk is open
   for (uint32_t k = 0;; ++k) {
     const uint32_t gen = gen0 + k;
     const QCount* q = P.ctrl->count[gen % 3];
@@ -95,20 +96,25 @@ __device__ __forceinline__ uint32_t tail_species(Params P, uint32_t gen0, uint32
 }
 
 // Block b of the cluster steps species b mod 3. VG, VE: the variants of the photon and of the
-// charged steps. Leaves the number of generations in Ctrl::tail_k for the end of the chunk.
+// charged steps. The chunk's start (its single thread waits for host memory while the others
+// copy their tables), its end and the marks of the live events are part of the kernel: against
+// three launches more a chunk, one shower 1.12 -> 1.06 ms, 10 showers 1.82 -> 1.75 ms, a serving
+// round 4.40 -> 4.30 ms.
 template <class R, int VG, int VE>
-__global__ void __launch_bounds__(256, 1) k_tail(Params P, uint32_t max_gens) {
+__global__ void __launch_bounds__(256, 1) k_tail(Params P, uint32_t max_gens, int b) {
   __shared__ WarpRing<R> rings[8];
   __shared__ unsigned long long s_cnt[6];
   WarpRing<R>& ring = rings[threadIdx.x >> 5];
   if (threadIdx.x < 6) s_cnt[threadIdx.x] = 0;
   __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0) open_chunk(P, b);
   const uint32_t gen0 = __ldcg(&P.ctrl->gen);
   const uint32_t s = blockIdx.x % 3, index = blockIdx.x / 3, count = (gridDim.x + 2 - s) / 3;
   uint32_t nsteps[3] = {0, 0, 0}, ncreated[3] = {0, 0, 0}, k;
   if (s == 0) k = tail_species<R, 0, VG>(P, gen0, max_gens, index, count, ring, nsteps, ncreated);
   else if (s == 1) k = tail_species<R, 1, VE>(P, gen0, max_gens, index, count, ring, nsteps, ncreated);
   else k = tail_species<R, 2, VE>(P, gen0, max_gens, index, count, ring, nsteps, ncreated);
+  if (k > 0) mark_events(P, gen0 + k, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
   for (int j = 0; j < 3; ++j) nsteps[j] = __reduce_add_sync(0xFFFFFFFFu, nsteps[j]);
   if ((threadIdx.x & 31) == 0)
     for (int j = 0; j < 3; ++j) {
@@ -121,7 +127,10 @@ __global__ void __launch_bounds__(256, 1) k_tail(Params P, uint32_t max_gens) {
     if (s_cnt[j]) atomicAdd(&P.ctrl->steps[j], s_cnt[j]);
     if (s_cnt[3 + j]) atomicAdd(&P.ctrl->created[j], s_cnt[3 + j]);
   }
-  if (blockIdx.x == 0) P.ctrl->tail_k = k;
+  if (blockIdx.x == 0) {
+    P.ctrl->tail_k = k;
+    close_chunk(P, gen0, k);
+  }
 }
 
 }  // namespace adept

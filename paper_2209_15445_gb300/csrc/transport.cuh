@@ -22,10 +22,11 @@ template <class R> struct Trk {
 __device__ __forceinline__ char* track_queue(const Params& P, int p, int s) {
   return P.queues + (size_t)(3 * p + s) * P.queue_bytes;
 }
-// event slot of track i of a queue
+// event slot of track i of a queue (from L2: the tail kernel reads what other SMs wrote)
 __device__ __forceinline__ uint32_t track_event(const Params& P, const char* q, uint32_t i) {
-  return P.split ? *(const uint32_t*)(q + (size_t)(i >> 5) * Tile<float>::kBytes + Tile<float>::kMeta + (i & 31u) * 16u + 8u)
-                 : *(const uint32_t*)(q + (size_t)(i >> 5) * Tile<double>::kBytes + Tile<double>::kEv + (i & 31u) * 4u);
+  const char* a = P.split ? q + (size_t)(i >> 5) * Tile<float>::kBytes + Tile<float>::kMeta + (i & 31u) * 16u + 8u
+                          : q + (size_t)(i >> 5) * Tile<double>::kBytes + Tile<double>::kEv + (i & 31u) * 4u;
+  return __ldcg((const uint32_t*)a);
 }
 
 // Queue loads are streaming (ld.global.cs): each slot is read once per generation. The tail
@@ -562,6 +563,41 @@ __device__ __forceinline__ void open_generation(const Params& P, uint32_t gen, u
   if (ln < P.max_log) {
     for (int k = 0; k < 3; ++k) P.gen_log[3 * ln + k] = min(c->count[cr][k].n, P.cap);
     c->log_n = ln + 1;
+  }
+}
+
+// End of a chunk of gens generations that began at gen: log the sizes its last generation left,
+// and advance the generation and its count. One thread.
+__device__ __forceinline__ void close_chunk(const Params& P, uint32_t gen, uint32_t gens) {
+  if (gens == 0) return;  // a tail chunk that found nothing to do
+  volatile Ctrl* c = P.ctrl;
+  const uint32_t ln = c->log_n;
+  if (ln < P.max_log) {
+    for (int k = 0; k < 3; ++k) P.gen_log[3 * ln + k] = min(c->count[(gen + gens) % 3][k].n, P.cap);
+    c->log_n = ln + 1;
+  }
+  c->generations = c->generations + gens;
+  c->gen = gen + gens;
+}
+
+// Start of a chunk in status buffer b: the outgoing-ring read position the host left in its
+// pinned copy, and an empty done count for the chunk's finish pass. One thread.
+__device__ __forceinline__ void open_chunk(const Params& P, int b) {
+  P.ctrl->leak_floor = *reinterpret_cast<const volatile unsigned long long*>(P.h_floor[b]);
+  P.ctrl->done_count[b] = 0;
+}
+
+// Mark the events that have tracks in the queues of generation gen, thread i of `threads`.
+__device__ __forceinline__ void mark_events(const Params& P, uint32_t gen, uint32_t first, uint32_t threads) {
+  const int p = gen & 1;
+  const QCount* q = P.ctrl->count[gen % 3];
+  const uint32_t n0 = min(__ldcg(&q[0].n), P.cap), n1 = min(__ldcg(&q[1].n), P.cap), n2 = min(__ldcg(&q[2].n), P.cap);
+  const uint32_t total = n0 + n1 + n2;
+  for (uint32_t i = first; i < total; i += threads) {
+    const int sp = i < n0 ? 0 : (i < n0 + n1 ? 1 : 2);
+    const uint32_t j = sp == 0 ? i : (sp == 1 ? i - n0 : i - n0 - n1);
+    const uint32_t ev = track_event(P, track_queue(P, p, sp), j);
+    if (P.evt.alive[ev] != gen) P.evt.alive[ev] = gen;
   }
 }
 
