@@ -168,7 +168,7 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
   const R tcut = (R)P.tcut;
   const R Er = to_r<R>(t.E);
   Stream<R> rs(P, __ldg(P.evt.key + t.ev), t.id, step);
-  if (Er < tcut) {
+  if (pos_lt(Er, tcut)) {
     dep = t.E;
     if (S == 2) { proc = 3; return kInteract; }  // annihilates at rest in phase B
     return kDead;
@@ -201,23 +201,24 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
       sg2 = lerp_rec<R>(rec, 4, tt);
     }
   }
-  sg0 = sg0 < (R)0 ? (R)0 : sg0;
-  sg1 = sg1 < (R)0 ? (R)0 : sg1;
-  sg2 = sg2 < (R)0 ? (R)0 : sg2;
+  sg0 = not_negative(sg0);
+  sg1 = not_negative(sg1);
+  sg2 = not_negative(sg2);
   const R stot = sg0 + sg1 + sg2;
   // S3/S4: sampled interaction length and the range-based step limit
-  R s_phys = stot > (R)0 ? M<R>::fdiv(-M<R>::flog(u0), stot) : M<R>::big();
+  R s_phys = is_positive(stot) ? M<R>::fdiv(-M<R>::flog(u0), stot) : M<R>::big();
   constexpr bool CH = (V & 1) != 0, PH = (V & 2) != 0 && S != 0;
   const bool msc = PH && (P.physics & 1u) != 0, fluct = PH && (P.physics & 2u) != 0;
   bool limited = false;  // the step limit, not the sampled interaction length, ends the step
   if (q != 0 && m >= 0) {
-    R smax = (Rr <= (R)kRhoF) ? Rr : ((R)kAlphaR * Rr > (R)kRhoF ? (R)kAlphaR * Rr : (R)kRhoF);
+    const R part = (R)kAlphaR * Rr;
+    R smax = pos_le(Rr, (R)kRhoF) ? Rr : (pos_lt((R)kRhoF, part) ? part : (R)kRhoF);
     if (PH && msc) {  // multiple-scattering step limit
       const R fR = (R)P.msc_f * Rr;
       const R sm = fR > (R)0.01 ? fR : (R)0.01;
       if (sm < smax) smax = sm;
     }
-    if (smax < s_phys) { s_phys = smax; limited = true; }
+    if (pos_lt(smax, s_phys)) { s_phys = smax; limited = true; }
   }
   // S5/S6: distance to the boundary along the straight line or helix
   int next;
@@ -239,7 +240,7 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
   } else {
     const R s_geom = field ? helix_distance<R, F>(P.geo, P.field_T, t.E, q, t.x, t.y, t.z, t.u, vol, &next)
                            : straight_distance<R, F>(P.geo, t.x, t.y, t.z, t.u, vol, &next);
-    boundary = s_geom <= s_phys;
+    boundary = pos_le(s_geom, s_phys);
     s = boundary ? s_geom : s_phys;
     if (field) {
       helix_move<R, F>(P.field_T, t.E, q, s, &t.x, &t.y, &t.z, t.u);
@@ -264,10 +265,10 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
   // that mean for a track that survives the mean loss
   if (q != 0 && m >= 0) {
     R Epr = 0;
-    if (s < Rr)
+    if (pos_lt(s, Rr))
       Epr = inverse_range<R>(range_nodes<R>(P.tab, S == 2) + m * kNNode, range_index<R>(P.tab, S == 2) + m * kRangeKeys,
                              Rr - s);
-    double Ep = (Epr > Er) ? t.E : to_d<R>(Epr);
+    double Ep = pos_lt(Er, Epr) ? t.E : to_d<R>(Epr);
     if constexpr (PH) {
       if (fluct && s < Rr && Ep >= P.tcut) {
         const R xi = (R)(kTwoPiRe2Me * __ldg(&P.mat[m].n_el));
@@ -278,7 +279,7 @@ __device__ __forceinline__ int step_transport(const Params& P, Trk<R>& t, Ixn<R>
     }
     dep += t.E - Ep;
     t.E = Ep;
-    if (Epr < tcut) {
+    if (pos_lt(Epr, tcut)) {
       dep += t.E;
       t.E = 0.0;
       if (S == 2) { proc = 3; return kInteract; }  // annihilates at rest in phase B
