@@ -15,7 +15,7 @@
 // 2.34 -> 2.13 ms, 100 showers 3.15 -> 2.84 ms, a round of 16 serving requests 5.15 -> 4.56 ms,
 // 1500 barrel primaries with chords, which leave a few tracks looping for 10,000 generations,
 // 345 -> 255 ms. What bounds it now: the dependent chain of one pass (a track's load, its step,
-// its interaction, its append), about 6 us, and 0.3 us of barrier.
+// its interaction, its append), about 4.5 us, and 0.3 us of barrier.
 // Species by block: a block's loop then holds one species' step, and nothing spills.
 #pragma once
 #include <type_traits>
@@ -89,8 +89,15 @@ __device__ __forceinline__ uint32_t tail_species(Params P, uint32_t gen0, uint32
     const uint32_t live = n[0] + n[1] + n[2];
     if (live == 0 || live >= P.tail_exit || k == max_gens) return k;
     if (blockIdx.x == 0 && threadIdx.x == 0) open_generation(P, gen, k);
-    run_tiles<R, S, V, true>(P, gen & 1, (gen + 1) % 3, (threadIdx.x >> 5) * count + index, (n[S] + 31) >> 5, count * wpb, n[S],
-                       ring, nsteps, ncreated);
+    // as few tracks a warp as the warps allow: lanes on different paths of the step (the chord
+    // and the bisection loops, the processes) run one after the other. Against full tiles, one
+    // 10 GeV shower 1.06 -> 1.00 ms, 1500 barrel primaries with chords 184.5 -> 135 ms, 10 FP64
+    // showers 6.57 -> 6.50 ms.
+    const uint32_t warps = count * wpb;
+    uint32_t shift = 0;
+    while (shift < 5u && (n[S] >> shift) > warps) ++shift;
+    run_tiles<R, S, V, true>(P, gen & 1, (gen + 1) % 3, (threadIdx.x >> 5) * count + index, (n[S] + (1u << shift) - 1u) >> shift,
+                             count * wpb, n[S], ring, nsteps, ncreated, shift);
     cluster_sync();
   }
 }

@@ -35,7 +35,7 @@ __device__ __forceinline__ uint32_t track_event(const Params& P, const char* q, 
 template <bool L2, class T> __device__ __forceinline__ T load_stream(const T* p) { return L2 ? __ldcg(p) : __ldcs(p); }
 template <bool L2>
 __device__ __forceinline__ void load_track(const char* q, uint32_t tile, uint32_t lane, Trk<double>& t) {
-  using L = Tile<double>;
+  using L = Tile<double>;  // lane: the track's place in its tile
   const char* a = q + (size_t)tile * L::kBytes;
   const double* d = (const double*)a + lane;
   const uint32_t* w = (const uint32_t*)(a + L::kEv) + lane;
@@ -474,7 +474,8 @@ __device__ __forceinline__ void prefetch_tile(const char* q, uint32_t tile, uint
 // misses).
 template <class R, int S, int V = 0, bool L2 = false>
 __device__ __forceinline__ void run_tiles(const Params& P, int p, int cw, uint32_t tile, uint32_t tiles, uint32_t stride,
-                                          uint32_t n, WarpRing<R>& ring, uint32_t* nsteps, uint32_t* ncreated) {
+                                          uint32_t n, WarpRing<R>& ring, uint32_t* nsteps, uint32_t* ncreated,
+                                          uint32_t shift = 5) {
   const uint32_t lane = threadIdx.x & 31;
   uint32_t head = 0, tail = 0;
   for (;;) {
@@ -490,11 +491,12 @@ __device__ __forceinline__ void run_tiles(const Params& P, int p, int cw, uint32
     int outcome = kDead, proc = 0, bin = -1;
     double dep = 0.0;
     if (phase_a) {
-      const uint32_t i = (tile << 5) + lane;
-      const bool active = i < n;
+      // (only the tail kernel takes smaller tiles: 2^shift tracks)
+      const uint32_t i = L2 ? (tile << shift) + lane : (tile << 5) + lane;
+      const bool active = L2 ? (lane >> shift) == 0u && i < n : i < n;
       const char* q = track_queue(P, p, S);
-      if (active) load_track<L2>(q, tile, lane, t);
-      if (tile + stride < tiles) prefetch_tile<R>(q, tile + stride, lane);
+      if (active) load_track<L2>(q, L2 ? i >> 5 : tile, L2 ? i & 31u : lane, t);
+      if (!L2 && tile + stride < tiles) prefetch_tile<R>(q, tile + stride, lane);
       if (active) outcome = step_transport<R, S, V>(P, t, sec, dep, bin, pstep, proc);
       nsteps[S] += active ? 1u : 0u;  // per lane; reduced over the warp at the end
     } else if (lane < c) {
