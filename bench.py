@@ -45,7 +45,7 @@ TRACK_BYTES_SPLIT = 64  # x,y,z f64 + direction 3 f32 + E f64 + id u64 + event, 
 # for the split form, profiles/transport_kernels_10gev_e_showers_fp64_gen60_full.md for the
 # plain FP64 form); valid while the kernel sources hash to NCU_SRC_HASH, null otherwise
 NCU_BYTES_PER_STEP = {1: 107.7, 0: 131.9}
-NCU_SRC_HASH = "953b78d11a1d49f9"
+NCU_SRC_HASH = "aed5ce0b28b4b9ad"
 
 
 def kernel_src_hash() -> str:
