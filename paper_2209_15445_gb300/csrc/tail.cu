@@ -34,6 +34,9 @@ static const void* tail_fn(const Params& P, int precision, bool fused) {
   return precision ? tail_fn<float>(transport_variant(P), fused) : tail_fn<double>(transport_variant(P), fused);
 }
 
+// The limit on dynamic shared memory belongs to the kernel, which every context of the process on
+// this device launches, each with its own tables: it is set to the most there is, whatever this
+// context needs, so that no context takes it from another and inits at the same time agree.
 uint32_t tail_shared_bytes(const Params& P, int precision, bool fused) {
   uint32_t n = 0;
   for (int s = 0; s < 3; ++s) n = std::max(n, precision ? tail_units<float>(P, s) : tail_units<double>(P, s));
@@ -43,7 +46,7 @@ uint32_t tail_shared_bytes(const Params& P, int precision, bool fused) {
   if (cudaFuncGetAttributes(&fa, fn) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
       16u * n + fa.sharedSizeBytes <= (size_t)most &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(16u * n)) == cudaSuccess)
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes) == cudaSuccess)
     return 16u * n;
   (void)cudaGetLastError();
   return 0;  // too many materials or volumes: read where they are
