@@ -355,15 +355,15 @@ int adept_raytrace(adept_ctx* ctx, int32_t prec, const double cam[11], int32_t n
  *               pair, photo), e- (dedx, range, ioni, brem), e+ (dedx, range, ioni, brem,
  *               annihilation) at the 289 grid energies (zeros for vacuum);
  *   dev_cuts:   caller-owned device memory, [n_materials][2] doubles (e-/e+ cut, gamma cut).
- * Needs no context and allocates nothing: its working rows (ADEPT_NOALLOC_MAX_MATERIALS x
- * 17 x 289 doubles, 157 KB) are a static device array that every GPU loading the library
- * holds until exit. The first call on a device looks up that array's device address with the
- * device current; make that first call before any stream capture. Work is queued on stream
- * (a cudaStream_t; results are ready when the stream reaches it). Every call shares the
- * array, so calls that overlap on the GPU (other streams, other threads) race; serialise
- * them. Returns ADEPT_EINVAL for a null pointer, a bad material or a compound (single
- * elements only), a non-positive cut or n_materials outside 1..ADEPT_NOALLOC_MAX_MATERIALS,
- * ADEPT_ECUDA if the launch fails. */
+ * Needs no context and allocates nothing: its working rows (ADEPT_NOALLOC_MAX_MATERIALS x 17 x
+ * 289 doubles and the materials' constants, 158 KB) are a static device array that every GPU
+ * loading the library holds until exit. The first call on a device looks up that array's
+ * device address with the device current; make that first call before any stream capture. Work
+ * is queued on stream (a cudaStream_t; results are ready when the stream reaches it). Every
+ * call shares the array, so calls on streams that overlap on the GPU race; serialise them.
+ * Calls of several threads on one stream follow one another. Returns ADEPT_EINVAL for a null
+ * pointer, a bad material or a compound (single elements only), a non-positive cut or
+ * n_materials outside 1..ADEPT_NOALLOC_MAX_MATERIALS, ADEPT_ECUDA if the launch fails. */
 #define ADEPT_NOALLOC_MAX_MATERIALS 4
 int adept_build_tables_noalloc(const adept_material* materials, int32_t n_materials, double range_cut_mm,
                                double* dev_tables, double* dev_cuts, void* stream);

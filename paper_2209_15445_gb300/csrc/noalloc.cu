@@ -16,10 +16,10 @@ namespace {
 constexpr int kRows = V_NROW + B_NROW;
 constexpr int kNoAllocMat = ADEPT_NOALLOC_MAX_MATERIALS;
 
-// Working rows and material constants of every call, on every device that loads the library
-// (held until exit): kNoAllocMat x 17 x 289 doubles = 157 KB. Calls share it; each call writes
-// every word it reads before reading it, so nothing needs clearing, but calls that overlap on
-// the GPU race on it.
+// Working rows (kNoAllocMat x 17 x 289 doubles) and material constants of every call, 158 KB on
+// every device that loads the library (held until exit). Calls share it; each call writes every
+// word it reads before reading it, so nothing needs clearing, but calls that overlap on the GPU
+// race on it.
 struct Scratch {
   double rows[kNoAllocMat * kRows * kNNode];
   MatDev mats[kNoAllocMat];
@@ -53,18 +53,17 @@ extern "C" int adept_build_tables_noalloc(const adept_material* materials, int32
   }
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return ADEPT_ECUDA;
-  Scratch* scratch;
-  {
+  // held until the last of the call's four launches is queued: between two of them no call of
+  // another thread on the same stream may queue its own, which write the same scratch
+  std::lock_guard<std::mutex> lk(g_mu);
+  if (!g_ptr[dev]) {
     // the array's device address, once per device with that device current; host code
     // cannot use the symbol itself (it names a host-side stand-in)
-    std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_ptr[dev]) {
-      void* p = nullptr;
-      if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return ADEPT_ECUDA;
-      g_ptr[dev] = static_cast<Scratch*>(p);
-    }
-    scratch = g_ptr[dev];
+    void* p = nullptr;
+    if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return ADEPT_ECUDA;
+    g_ptr[dev] = static_cast<Scratch*>(p);
   }
+  Scratch* const scratch = g_ptr[dev];
   const TableRows r{scratch->rows, (size_t)kRows * kNNode, scratch->rows + V_NROW * kNNode, (size_t)kRows * kNNode,
                     dev_cuts, dev_cuts + 1, 2, dev_tables};
   return launch_table_rows(in, n_materials, range_cut_mm, scratch->mats, r, static_cast<cudaStream_t>(stream)) == cudaSuccess
