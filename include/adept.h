@@ -163,13 +163,18 @@ typedef struct {
                                  next chunk is a tail chunk: one kernel that runs the generations
                                  in one launch and stops as soon as the queues are empty, once
                                  twice as many tracks are live, or after graph_generations
-                                 generations; < 0: never [16384] */
+                                 generations; < 0: never [16384]. Contexts with the
+                                 optional physics have no tail chunks, and those with
+                                 ADEPT_FLAG_TIME_SPECIES only once fewer tracks are live than an
+                                 eighth of the peak since the queues were last empty */
 } adept_options;
 
 /* adept_options.flags: time every generation (its three transport kernels, from the fork to
- * the join) with CUDA events recorded inside the captured graphs; totals in adept_stats */
+ * the join) with CUDA events recorded inside the captured graphs, and the generations of a tail
+ * chunk together; totals in adept_stats */
 #define ADEPT_FLAG_TIME_STEPS 1
-/* also time each species kernel separately (two more events per generation) */
+/* also time each species kernel separately (two more events per generation; but for tail
+ * chunks, whose one kernel steps all three, and which only take the decay then) */
 #define ADEPT_FLAG_TIME_SPECIES 4
 /* histogram the length of every step (validation; costs one atomic per step; runs kernels
  * compiled with the histogram, so not with fused = 1 or field_max_iterations > 0, which
@@ -217,9 +222,9 @@ typedef struct {
   uint64_t step_launches; /* generations timed (ADEPT_FLAG_TIME_STEPS or _SPECIES) */
   double step_kernel_ms;  /* summed CUDA-event durations of their generations (fork to the
                              end of the last of the three concurrent species kernels, or the
-                             fused kernel) */
+                             fused kernel; the tail kernel from start to end) */
   double species_ms[3];   /* per species kernel (gamma, e-, e+): fork to its end, summed
-                             (ADEPT_FLAG_TIME_SPECIES only) */
+                             (ADEPT_FLAG_TIME_SPECIES only, without the tail kernel) */
 } adept_stats;
 
 /* Create a context: validates geometry and materials, lays out dev_arena (device memory

@@ -154,6 +154,7 @@ struct adept_ctx {
   int tail_blocks = 0;
   bool tail[2] = {false, false};  // the chunk queued in buffer b is a tail chunk
   uint64_t last_live = 0;         // live tracks at the end of the last chunk read back
+  uint64_t peak_live = 0;         // most live tracks read back since the queues were last empty
   // estimated peak tracks (tracks_per_MeV x energy, plus the primaries) of the requests
   // admitted so far; its value when chunk b was launched; and the value behind last_live
   uint64_t admit_est = 0, admit_mark[2] = {0, 0}, admit_seen = 0;
@@ -776,6 +777,9 @@ static int capture_graph(adept_ctx* c, int gens, int b) {
   return ADEPT_OK;
 }
 
+// ADEPT_FLAG_TIME_SPECIES: the part of the peak below which a population is in its decay
+constexpr uint64_t kTailDecay = 8;
+
 // Queue one chunk of generations and the copy of its status into buffer b; returns at once.
 static int launch_chunk(adept_ctx* c, int b) {
   const int G = c->opt.graph_generations;
@@ -788,10 +792,15 @@ static int launch_chunk(adept_ctx* c, int b) {
     if (rc) return rc;
   }
   const uint64_t live = c->last_live + (c->admit_est - c->admit_seen);
-  c->tail[b] = G > 0 && live < (uint64_t)c->tail_tracks;
+  // (the tail kernel's time has no species: with the times per species it takes the decay only,
+  // 30 showers of 2 GeV 2.06 ms, where fixed chunks and their empty generations took 2.53)
+  c->tail[b] = G > 0 && live < (uint64_t)c->tail_tracks && (!timing_species(c) || live * kTailDecay < c->peak_live);
   c->admit_mark[b] = c->admit_est;
   if (c->tail[b]) {
+    cudaEvent_t* ev = timing(c) ? c->ev.data() + 4 * gens * b : nullptr;
+    if (ev) CK(cudaEventRecord(ev[0], c->stream));
     CK(launch_tail(c->P, c->opt.precision, c->opt.fused != 0, c->tail_blocks, (uint32_t)gens, b, c->stream));
+    if (ev) CK(cudaEventRecord(ev[1], c->stream));
     CK(launch_done(c->P, b, c->slot_end, c->stream));
     c->stats.launches += 2;
   } else if (G > 0) {
@@ -813,10 +822,19 @@ static int launch_chunk(adept_ctx* c, int b) {
 // Wait for chunk b and account its timing events.
 static int wait_chunk(adept_ctx* c, int b) {
   CK(cudaEventSynchronize(c->status_ev[b]));
-  if (timing(c) && !c->tail[b]) {  // tail chunks are not timed
+  if (timing(c)) {
     const int G = c->opt.graph_generations;
     const int gens = G > 0 ? G : 1;
     const cudaEvent_t* ev = c->ev.data() + 4 * gens * b;
+    if (c->tail[b]) {  // timed as one, over the generations it ran
+      const uint32_t ran = c->h_ctrl[b]->tail_k;
+      if (ran == 0) return ADEPT_OK;
+      float ms = 0.f;
+      CK(cudaEventElapsedTime(&ms, ev[0], ev[1]));
+      c->stats.step_kernel_ms += ms;
+      c->stats.step_launches += ran;
+      return ADEPT_OK;
+    }
     // concurrent species kernels: each one's time from the generation's fork to its end;
     // the generation's time is the longest of the three
     for (int k = 0; k < gens; ++k) {
@@ -1039,6 +1057,7 @@ extern "C" int adept_transport(adept_ctx* c, uint64_t timeout_us) {
     done.assign(c->h_done[b], c->h_done[b] + nd);
     const uint32_t live = h.count[h.gen % 3][0].n + h.count[h.gen % 3][1].n + h.count[h.gen % 3][2].n;
     c->last_live = live;
+    c->peak_live = live ? std::max<uint64_t>(c->peak_live, live) : 0;
     c->admit_seen = c->admit_mark[b];
     // While tracks are live and no request waits for admission, relaunch buffer b at once, so
     // that the host's processing of this status (outgoing particles, finished events) overlaps

@@ -98,7 +98,7 @@ struct Ctrl {
   uint32_t done_count[2];     // events found finished by the finish pass of a chunk (per buffer)
   uint32_t log_n;             // rows written to the generation log
   uint32_t error;             // first device-detected error code (0 = none)
-  uint32_t tail_k;            // generations the last tail chunk ran
+  uint32_t tail_k;            // generations the last tail chunk ran (timed together)
   uint32_t finish_ticket;     // blocks of the finish pass that have ended (the last one resets it)
   uint32_t pad[2];
   unsigned long long steps[3];
