@@ -335,6 +335,13 @@ int adept_probe_continuous(adept_ctx* ctx, int32_t which, int32_t species, int32
 int adept_probe_chord(adept_ctx* ctx, int32_t prec, const double* host_pos, const double* host_dir,
                       const int32_t* host_vol, const double* host_T, const int32_t* host_charge,
                       const double* host_s_phys, size_t n, double* host_out);
+/*  - quotient: for n pairs, x / d as the split form takes its quotients by one number, and by
+ *    the division: 2 floats per pair.
+ *  - chord_direction: for n vectors v[3n], the length and the direction of a chord as the
+ *    split form's propagator takes them, and from the square root and the divisions: 2 x 4
+ *    doubles per vector. */
+int adept_probe_quotient(adept_ctx* ctx, const float* host_d, const float* host_x, size_t n, float* host_out);
+int adept_probe_chord_direction(adept_ctx* ctx, const double* host_v, size_t n, double* host_out);
 
 /* Ray-traced image of the geometry (paper Sec. 2.1: navigation validated on ray-traced
  * images, GPU against CPU and single against double precision). Orthographic camera

@@ -146,6 +146,8 @@ def load(path: str = LIB_PATH):
             "adept_probe_continuous": [vp, i32, i32, i32, i32, C.c_double, C.c_double, u32, sz, dp],
             "adept_raytrace": [vp, i32, dp, i32, i32, C.c_void_p, i32],
             "adept_probe_chord": [vp, i32, dp, dp, C.POINTER(C.c_int32), dp, C.POINTER(C.c_int32), dp, sz, dp],
+            "adept_probe_quotient": [vp, C.POINTER(C.c_float), C.POINTER(C.c_float), sz, C.POINTER(C.c_float)],
+            "adept_probe_chord_direction": [vp, dp, sz, dp],
             "adept_build_tables_noalloc": [C.POINTER(adept_material), i32, C.c_double, vp, vp, vp],
         }
         for name, args in sig.items():
@@ -338,6 +340,23 @@ def adept_probe_chord(h, prec, pos, d, vol, T, q, s_phys):
     rc = load().adept_probe_chord(h, prec, _dp(pos), _dp(d), vol.ctypes.data_as(i32p), _dp(T),
                                   q.ctypes.data_as(i32p), _dp(s_phys), n, _dp(out))
     return rc, out
+
+
+def adept_probe_quotient(h, d, x):
+    """(rc, quotients of the split form, quotients of the division)"""
+    d = np.ascontiguousarray(d, np.float32); x = np.ascontiguousarray(x, np.float32)
+    out = np.zeros((len(d), 2), np.float32)
+    fp = C.POINTER(C.c_float)
+    rc = load().adept_probe_quotient(h, d.ctypes.data_as(fp), x.ctypes.data_as(fp), len(d), out.ctypes.data_as(fp))
+    return rc, out[:, 0], out[:, 1]
+
+
+def adept_probe_chord_direction(h, v):
+    """(rc, (n, 4) length and direction of the split form's chords, the same by divisions)"""
+    v = np.ascontiguousarray(v, np.float64).reshape(-1, 3)
+    out = np.zeros((len(v), 2, 4))
+    rc = load().adept_probe_chord_direction(h, _dp(v), len(v), _dp(out))
+    return rc, out[:, 0], out[:, 1]
 
 
 def adept_probe_continuous(h, which, species, m, prec, T, s, event, n):

@@ -1456,6 +1456,34 @@ extern "C" int adept_probe_chord(adept_ctx* c, int32_t prec, const double* pos, 
   return ADEPT_OK;
 }
 
+extern "C" int adept_probe_quotient(adept_ctx* c, const float* d, const float* x, size_t n, float* out) {
+  if (!c || (n && (!d || !x || !out))) return ADEPT_EINVAL;
+  return probe_run(c, 8, 8, n, [&](size_t b, size_t k) {
+    float* dd = reinterpret_cast<float*>(c->probe);
+    float* dx = dd + k;
+    float* dout = dx + k;
+    CK(cudaMemcpyAsync(dd, d + b, 4 * k, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemcpyAsync(dx, x + b, 4 * k, cudaMemcpyHostToDevice, c->stream));
+    CK(launch_probe_quotient(dd, dx, (int)k, dout, c->stream));
+    CK(cudaMemcpyAsync(out + 2 * b, dout, 8 * k, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    return ADEPT_OK;
+  });
+}
+
+extern "C" int adept_probe_chord_direction(adept_ctx* c, const double* v, size_t n, double* out) {
+  if (!c || (n && (!v || !out))) return ADEPT_EINVAL;
+  return probe_run(c, 24, 64, n, [&](size_t b, size_t k) {
+    double* dv = reinterpret_cast<double*>(c->probe);
+    double* dout = dv + 3 * k;
+    CK(cudaMemcpyAsync(dv, v + 3 * b, 24 * k, cudaMemcpyHostToDevice, c->stream));
+    CK(launch_probe_chord_direction(dv, (int)k, dout, c->stream));
+    CK(cudaMemcpyAsync(out + 8 * b, dout, 64 * k, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    return ADEPT_OK;
+  });
+}
+
 extern "C" int adept_probe_continuous(adept_ctx* c, int32_t which, int32_t species, int32_t m, int32_t prec, double T,
                                       double s, uint32_t event, size_t n, double* host_out) {
   if (!c || which < 0 || which > 1 || (species != 1 && species != 2) || m < 0 || m >= c->n_mat ||

@@ -440,6 +440,39 @@ cudaError_t launch_probe_chord(const Params& P, int prec, const double* pos, con
   return cudaGetLastError();
 }
 
+// the split form's quotients, and beside each the division it stands for
+__global__ void k_probe_quotient(const float* d, const float* x, int n, float* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  out[2 * i] = Over<float>(d[i])(x[i]);
+  out[2 * i + 1] = __fdiv_rn(x[i], d[i]);
+}
+
+cudaError_t launch_probe_quotient(const float* d, const float* x, int n, float* out, cudaStream_t st) {
+  if (n > 0) k_probe_quotient<<<(n + 127) / 128, 128, 0, st>>>(d, x, n, out);
+  return cudaGetLastError();
+}
+
+// a chord's length and direction in the split form, and beside them those from the square root
+// and the divisions, cut the same way (all zero where the length is)
+__global__ void k_probe_chord_direction(const double* v, int n, double* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double dx = v[3 * i], dy = v[3 * i + 1], dz = v[3 * i + 2];
+  float Lf, f[3];
+  double Ld, d[3];
+  if (!chord_direction(dx, dy, dz, &Lf, f)) f[0] = f[1] = f[2] = 0.0f;
+  if (!chord_direction(dx, dy, dz, &Ld, d)) d[0] = d[1] = d[2] = 0.0;
+  double* o = out + 8 * (size_t)i;
+  o[0] = Lf; o[4] = to_r<float>(Ld);
+  for (int k = 0; k < 3; ++k) { o[1 + k] = f[k]; o[5 + k] = to_r<float>(d[k]); }
+}
+
+cudaError_t launch_probe_chord_direction(const double* v, int n, double* out, cudaStream_t st) {
+  if (n > 0) k_probe_chord_direction<<<(n + 127) / 128, 128, 0, st>>>(v, n, out);
+  return cudaGetLastError();
+}
+
 template <class R>
 __global__ void k_probe_sample(Params P, int which, int m, double E, uint32_t event, int n, double* out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;

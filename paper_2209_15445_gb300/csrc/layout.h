@@ -273,6 +273,8 @@ cudaError_t launch_raytrace(const Params& P, int prec, const RayCam& cam, int nx
                             double* out, cudaStream_t st);
 cudaError_t launch_probe_chord(const Params& P, int prec, const double* pos, const double* dir, const int* vol,
                                const double* T, const int* q, const double* s_phys, int n, double* out, cudaStream_t st);
+cudaError_t launch_probe_quotient(const float* d, const float* x, int n, float* out, cudaStream_t st);
+cudaError_t launch_probe_chord_direction(const double* v, int n, double* out, cudaStream_t st);
 cudaError_t launch_probe_continuous(const Params& P, int which, int species, int m, int prec, double T, double s,
                                     uint32_t event, int n, double* out, cudaStream_t st);
 // generation gen + gk of all species in one kernel
