@@ -205,6 +205,9 @@ cudaError_t launch_build_tables(const Params& P, const double* mat_in, int n_mat
 // (ms, by kTailTracks): 10 showers of 10 GeV 2.20 (4096), 2.13 (8192), 2.04 (16384), 2.38 with
 // fixed chunks; 100 showers 2.84, 2.84, 2.75, 3.15; a round of 16 serving requests 4.55, 4.56,
 // 4.62, 5.1. FP64, whose generations want more SMs: 10 showers 6.8 (512 to 2048), 8.4 (8192).
+// In a field the same line (barrel primaries in 3.8 T): 50 of them 3.74 (2048), 3.41 (12288),
+// 4.07 (fixed chunks); 100 in the fused form 3.13, 2.99, 3.28; with chords 60 13.6, 13.2, 14.7,
+// 1500 45.8, 45.7, 48.2, and with their loopers' 10,000 generations the same from 1024 to 12288.
 constexpr uint32_t kTailTracks = 12288, kTailTracksFp64 = 2048;
 cudaError_t launch_tail(const Params& P, int precision, bool fused, int blocks, uint32_t max_gens, int b, cudaStream_t st);
 // the bytes for Params::tail_shared, and then the blocks of its cluster (one a species in turn):
