@@ -45,7 +45,7 @@ TRACK_BYTES_SPLIT = 64  # x,y,z f64 + direction 3 f32 + E f64 + id u64 + event, 
 # for the split form, profiles/transport_kernels_10gev_e_showers_fp64_gen60_full.md for the
 # plain FP64 form); valid while the kernel sources hash to NCU_SRC_HASH, null otherwise
 NCU_BYTES_PER_STEP = {1: 107.7, 0: 131.9}
-NCU_SRC_HASH = "aed5ce0b28b4b9ad"
+NCU_SRC_HASH = "6b3fdc17254f6f11"
 
 
 def kernel_src_hash() -> str:
@@ -314,7 +314,7 @@ def run_ours(a):
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": (achieved / peak) if achieved else None, "traffic": traffic,
             "kernel": ("k_fused_generation<%s> (one launch = one generation, all species)" if tr.options.fused else
-                       "k_transport<%s, species> x3, concurrent (one launch = one generation: gamma, e+, e-)")
+                       "k_transport<%s, species> x3, concurrent, and k_tail (one launch = one generation: gamma, e+, e-)")
                       % ("float" if a.precision else "double"),
             "alg_bytes_per_launch": alg_bytes / kern_n if kern_n else None,
             "mean_launch_us": 1e3 * kern_ms / kern_n if kern_n else None,
